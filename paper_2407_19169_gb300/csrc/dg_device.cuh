@@ -364,21 +364,54 @@ __device__ __forceinline__ T pressure_of(const T* w, T gm1) {
   else return gm1 * (w[3] - T(0.5) * (w[1] * w[1] + w[2] * w[2]) / w[0]);
 }
 
-// Largest t in [0, 1] with p(ub + t (w - ub)) >= eps, by bisection (the admissible set is convex,
-// so p - eps changes sign once on the segment; p(ub) >= eps, p(w) < eps on entry).
+// Largest t in [0, top] with p(ub + t (w - ub)) >= eps; top if the pressure holds there. Pressure is a
+// concave function of the conservative state, so on the segment p - eps changes sign once (p(ub) >=
+// eps) and Newton's iteration from a failing point comes down to the root from the right without
+// passing it, quadratically (4 to 6 evaluations instead of the 30 (FP32) and 60 (FP64) of a bisection).
+// Rounding leaves it a few units in the last place on the failing side: from there t steps back, twice
+// as far each time, to the first point where the pressure holds. Both loops are bounded; t = 0 (the
+// average itself) always holds.
 template <int NV, class T>
-__device__ __noinline__ T pp_segment(const T* ub, const T* w, T eps, T gm1) {
-  T lo = T(0), hi = T(1);
-  const int iters = sizeof(T) == 8 ? 60 : 30;
-#pragma unroll 1
-  for (int it = 0; it < iters; ++it) {
-    const T mid = T(0.5) * (lo + hi);
+__device__ __forceinline__ T pp_segment(const T (&ub)[NV], const T (&w)[NV], T eps, T gm1, T top) {
+  T d[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) d[v] = w[v] - ub[v];
+  // p - eps at t, and its derivative
+  auto gap = [&](T t, T& slope) -> T {
     T x[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) x[v] = ub[v] + mid * (w[v] - ub[v]);
-    if (pressure_of<NV>(x, gm1) >= eps) lo = mid; else hi = mid;
+    for (int v = 0; v < NV; ++v) x[v] = ub[v] + t * d[v];
+    T mm = T(0), md = T(0);
+#pragma unroll
+    for (int v = 1; v < NV - 1; ++v) {
+      mm += x[v] * x[v];
+      md += x[v] * d[v];
+    }
+    const T inv = T(1) / x[0];
+    slope = gm1 * (d[NV - 1] - (md - T(0.5) * mm * inv * d[0]) * inv);
+    return gm1 * (x[NV - 1] - T(0.5) * mm / x[0]) - eps;
+  };
+  T t = top, slope;
+  T g = gap(t, slope);
+  const int iters = sizeof(T) == 8 ? 60 : 30;
+  const T ulp = sizeof(T) == 8 ? T(2.3e-16) : T(1.2e-7);
+#pragma unroll 1
+  for (int it = 0; it < iters && g < T(0); ++it) {
+    const T next = t - g / slope;
+    if (!(next < t * (T(1) - ulp)) || !(next > T(0))) break;   // converged, or no descent
+    t = next;
+    g = gap(t, slope);
   }
-  return lo;
+  T back = ulp;
+  const T from = t;
+#pragma unroll 1
+  for (int it = 0; it < iters && g < T(0); ++it) {
+    t = from * (T(1) - back);
+    if (!(t > T(0))) return T(0);
+    back += back;
+    g = gap(t, slope);
+  }
+  return g < T(0) ? T(0) : t;
 }
 
 // ---- storage of the FP32 form ---------------------------------------------------------------

@@ -452,8 +452,7 @@ struct Stage1D {
           w[v] = x;
         }
         if (pressure_of<NV>(w, gm1) < eps) {
-          const T t = pp_segment<NV>(ub, w, eps, gm1);
-          th2 = t < th2 ? t : th2;
+          th2 = pp_segment<NV>(ub, w, eps, gm1, th2);
         }
       }
       if (th2 < T(1)) {
