@@ -17,7 +17,7 @@ LIB = os.path.join(HERE, "libdgjf.so")
 # kernel and once for its dispatch tables, dg_batch.cu once for its host code and 1D kernels and once
 # per degree of its 2D kernels, so that the slow instantiations compile in parallel.
 UNITS = [(u, u.replace(".cu", ".o"), []) for u in
-         ["dg_api.cu", "aux.cu", "stage1d.cu", "dg_noalloc.cu", "dg_batch.cu", "probes.cu"]] + \
+         ["dg_api.cu", "aux.cu", "rate.cu", "stage1d.cu", "dg_noalloc.cu", "dg_batch.cu", "probes.cu"]] + \
         [("stage2d_units.cu", "stage2d_f%d_k%d.o" % (f, k), ["-DS2_FORM=%d" % f, "-DS2_K=%d" % k])
          for f in range(5) for k in (1, 2, 3)] + \
         [("stage2d_units.cu", "stage2d_dispatch.o", ["-DS2_DISPATCH"])] + \

@@ -64,6 +64,25 @@ inline void stage1d_consts(Stage1DArgs& a) {
   a.c0_lo = (float)(a.c0 - (double)a.c0_hi);
 }
 
+// Values of P_l at the positivity limiter's points in 1D (degree K), [point][l]: the Gauss points, both
+// ends and, for K = 3, the node 0 of the 3-point Gauss-Lobatto rule (Zhang and Shu's positivity of the
+// averages uses the Lobatto nodes with 2N - 3 >= k; for K = 2 the node 0 is a Gauss node already).
+__host__ __device__ constexpr int limiter_points1(int K) { return K + 3 + ((K >= 2 && K % 2 == 1) ? 1 : 0); }
+template <int K>
+__host__ __device__ constexpr double limiter_value1(int i, int l) {
+  return i <= K ? GaussRule<K + 1>::P(l, i < K + 1 ? i : 0)
+                : (i == K + 1 ? ((l & 1) ? -1.0 : 1.0) : (i == K + 2 ? 1.0 : GaussRule<1>::P(l, 0)));
+}
+template <int K, class T>
+constexpr carr<T, limiter_points1(K) * (K + 1)> limiter_values1() {
+  carr<T, limiter_points1(K) * (K + 1)> t{};
+  for (int i = 0; i < limiter_points1(K); ++i)
+    for (int l = 0; l <= K; ++l) t[i * (K + 1) + l] = (T)limiter_value1<K>(i, l);
+  return t;
+}
+template <int K, class T>
+__constant__ carr<T, limiter_points1(K) * (K + 1)> lim_table1 = limiter_values1<K, T>();
+
 // OE = true: the OEDG form of the damping (the kernel stores u~ unfiltered with the jump sums A_v(l)
 // and the reductions of OedgOut; the OEDG filter kernel applies the damping).
 // COH = true: state loads through L2 (Store), for the persistent batched kernel.
@@ -367,14 +386,8 @@ struct Stage1D {
     if constexpr (OE) oedg_reduce<NV>(a.oe, osum, omax, omin);
   }
 
-  // The limiter's points: the Gauss points, both ends and, for k = 3, the node 0 of the 3-point
-  // Gauss-Lobatto rule (Zhang and Shu's positivity of the averages uses the Lobatto nodes with
-  // 2N - 3 >= k; for k = 2 the node 0 is a Gauss node already). Value of P_l at point i.
-  static constexpr int NP_LIM = NQ + 2 + ((K >= 2 && NQ % 2 == 0) ? 1 : 0);
-  static __device__ __forceinline__ double lim_coef(int i, int l) {
-    constexpr carr<double, (K + 1) * NQ> GPT = TB::GP;
-    return i < NQ ? GPT[l * NQ + i] : (i == NQ ? ((l & 1) ? -1.0 : 1.0) : (i == NQ + 1 ? 1.0 : GaussRule<1>::P(l, 0)));
-  }
+  static constexpr int NP_LIM = limiter_points1(K);
+  static __device__ __forceinline__ double lim_coef(int i, int l) { return limiter_value1<K>(i, l); }
 
   // Max CFL rate beta / h over the positivity limiter's points of one cell: with the limiter on,
   // Zhang and Shu's positivity result for the averages needs the CFL bound on the wave speeds at
