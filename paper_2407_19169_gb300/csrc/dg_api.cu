@@ -257,9 +257,21 @@ int dgk::default_block_warps(const StageLauncher& L, int max_wpb) {
 
 static dg_status setup_launch(dg_solver* s, int tile_rows, int tile_warps) {
   if (s->dim == 1) {
+    s->nwarps1d = (s->mesh.nx + STRIP_OUT - 1) / STRIP_OUT;
+    // the whole step in one launch, unless a second kernel has to run between the stages
+    s->whole_step = !s->hybrid && !s->geom.oedg;
+    if (s->whole_step) {
+      s->L = step1d_launcher(s->k, s->eq, s->prec);
+      if (!s->L.launch) return DG_ERR_UNSUPPORTED;
+      const Step1DGrid g = step1d_grid(s->L, s->mesh.nx);
+      s->block = g.block;
+      s->grid = g.grid;
+      s->ntiles1d = g.tiles;
+      s->smem = 0;
+      return DG_OK;
+    }
     s->L = stage1d_launcher(s->k, s->eq, s->prec, s->geom.oedg != 0);
     if (!s->L.launch) return DG_ERR_UNSUPPORTED;
-    s->nwarps1d = (s->mesh.nx + STRIP_OUT - 1) / STRIP_OUT;
     s->block = 128;
     // at most 8 blocks of 4 warps per SM (64 registers a thread); warps loop over strips
     long long g1 = (s->nwarps1d + 3) / 4;
@@ -552,17 +564,15 @@ extern "C" dg_status dg_read_state(const dg_solver* cs, double* host, size_t n, 
   return DG_OK;
 }
 
-// Launch the three stages of one step starting from buffer parity p.
-static const double SO_C0[3] = {0.0, 0.75, 1.0 / 3.0};
-static const double SO_C1[3] = {1.0, 0.25, 2.0 / 3.0};
-
+// Launch one step starting from buffer parity p: its three stages, or in 1D the whole step at once.
 static cudaError_t launch_step(dg_solver* s, int p) {
   void* in = s->buf[p];
   void* nx = s->buf[1 - p];
   void* tmp = s->buf[2];
   const void* srcs[3] = {in, nx, tmp};
   void* dsts[3] = {nx, tmp, nx};
-  for (int st = 0; st < 3; ++st) {
+  const int stages = s->whole_step ? 1 : 3;
+  for (int st = 0; st < stages; ++st) {
     cudaError_t e;
     if (s->dim == 1) {
       Stage1DArgs a;
@@ -573,14 +583,14 @@ static cudaError_t launch_step(dg_solver* s, int p) {
       a.ncell = s->geom.ncell;
       a.h = s->geom.hx;
       a.bc = s->mesh.bc[0];
-      a.c0 = SO_C0[st];
-      a.c1 = SO_C1[st];
+      a.c0 = so_c0(st);
+      a.c1 = so_c1(st);
       a.stage = st;
       a.filter_on = s->filter_on;
       a.gamma = s->gamma;
       a.ax = s->ax;
       a.cfl = s->cfl;
-      a.nwarps = s->nwarps1d;
+      a.nwarps = s->whole_step ? s->ntiles1d : s->nwarps1d;
       a.positivity = s->positivity;
       a.hybrid = s->hybrid;
       a.hyb = s->hy;
@@ -600,8 +610,8 @@ static cudaError_t launch_step(dg_solver* s, int p) {
       a.hy = s->geom.hy;
       a.bcx = s->mesh.bc[0];
       a.bcy = s->mesh.bc[2];
-      a.c0 = SO_C0[st];
-      a.c1 = SO_C1[st];
+      a.c0 = so_c0(st);
+      a.c1 = so_c1(st);
       a.stage = st;
       a.filter_on = s->filter_on;
       a.gamma = s->gamma;

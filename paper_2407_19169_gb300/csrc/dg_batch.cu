@@ -32,8 +32,8 @@ struct BatchInst {
   int nx, ny, bcx, bcy, H, nstrips, nchunks, filter_on, positivity;
   double hx, hy, gamma, ax, ay, cfl;
   // 1D mesh constants from the host (stage1d_consts)
-  double inv_h_d, scl_d, wpow_d[4];
-  float inv_h_f, scl_f, wpow_f[4];
+  double inv_h_d;
+  float inv_h_f;
   // 2D mesh constants from the host (stage2d_consts)
   Consts2D<float> cf;
   Consts2D<double> cd;
@@ -191,21 +191,13 @@ __global__ void __launch_bounds__(256) batch1d_kernel(const BatchArgs b) {
     a.hyb = HybridOut{};
     a.sc = I.sc;
     a.inv_h_d = I.inv_h_d;
-    a.scl_d = I.scl_d;
     a.inv_h_f = I.inv_h_f;
-    a.scl_f = I.scl_f;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      a.wpow_d[m] = I.wpow_d[m];
-      a.wpow_f[m] = I.wpow_f[m];
-    }
     a.c0_hi = b.c0_hi;
     a.c0_lo = b.c0_lo;
-    double r = 0.0;
-    T rt = T(0);
+    T speed = T(0);
     bool ok = true;
-    S::item(a, dt, w - I.item0, r, rt, ok);
-    if constexpr (PR::MIXED) r = (double)rt;
+    S::item(a, dt, w - I.item0, speed, ok);
+    const double r = (double)speed * I.inv_h_d;
     racc = (r > racc || r != r) ? r : racc;
     okacc = okacc && ok;
   }
@@ -229,7 +221,6 @@ __global__ void batch_begin_kernel(const BatchInst* inst, int n) {
   const bool last = (t + dtc >= T);
   sc->dt = last ? T - t : dtc;
   sc->is_last = last ? 1u : 0u;
-  sc->rate_bits[(step + 1) & 1] = 0ull;
 }
 
 // Per-instance step advance at the end of a step (the single-solve last-block rule).
@@ -242,6 +233,7 @@ __global__ void batch_end_kernel(const BatchInst* inst, int n) {
   const long long st = sc->step + 1;
   sc->t = tn;
   sc->step = st;
+  sc->rate_bits[(st + 1) & 1] = 0ull;     // the slot of the next step
   sc->done = (tn >= sc->T_end || st >= sc->max_step) ? 1u : 0u;
 }
 
@@ -313,6 +305,7 @@ __device__ __forceinline__ void persist_step_advance(const BatchInst& I, bool ne
   const long long st = sc->step + 1;
   sc->t = tn;
   sc->step = st;
+  sc->rate_bits[(st + 1) & 1] = 0ull;     // the slot of the next step
   const bool done = (tn >= sc->T_end || st >= sc->max_step);
   sc->done = done ? 1u : 0u;
   if (done || !next) return;
@@ -325,7 +318,6 @@ __device__ __forceinline__ void persist_step_advance(const BatchInst& I, bool ne
   const bool last = (tn + dtc >= T);
   sc->dt = last ? T - tn : dtc;
   sc->is_last = last ? 1u : 0u;
-  sc->rate_bits[(st + 1) & 1] = 0ull;
 }
 
 // Arrival of one finished (or skipped) item; the last item of an instance's stage releases it.
@@ -452,24 +444,16 @@ __global__ void __launch_bounds__(256) persist1d_kernel(const PersistArgs P) {
       a.hyb = HybridOut{};
       a.sc = I.sc;
       a.inv_h_d = I.inv_h_d;
-      a.scl_d = I.scl_d;
       a.inv_h_f = I.inv_h_f;
-      a.scl_f = I.scl_f;
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        a.wpow_d[m] = I.wpow_d[m];
-        a.wpow_f[m] = I.wpow_f[m];
-      }
       {
         const double c0 = a.c0;
         a.c0_hi = (float)c0;
         a.c0_lo = (float)(c0 - (double)a.c0_hi);
       }
-      double r = 0.0;
-      T rt = T(0);
+      T speed = T(0);
       bool ok = true;
-      S::item(a, dt, w - I.item0, r, rt, ok);
-      item_end(I, stage, step, (double)rt, ok);
+      S::item(a, dt, w - I.item0, speed, ok);
+      item_end(I, stage, step, (double)speed * I.inv_h_d, ok);
     }
     persist_arrive(P, I, C, phase);
   }
@@ -675,13 +659,7 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
         t.h = s->geom.hx;
         stage1d_consts(t);
         I.inv_h_d = t.inv_h_d;
-        I.scl_d = t.scl_d;
         I.inv_h_f = t.inv_h_f;
-        I.scl_f = t.scl_f;
-        for (int m = 0; m < 4; ++m) {
-          I.wpow_d[m] = t.wpow_d[m];
-          I.wpow_f[m] = t.wpow_f[m];
-        }
       }
       cls_items[c] += (long long)I.nstrips * I.nchunks;
       host.push_back(I);

@@ -38,6 +38,8 @@ struct DevScalars {
   unsigned int err;               // ERRB_* bits; stage kernels do nothing
   unsigned int blocks_done;       // last-block counter of the final stage
   unsigned int is_last;           // current step is clipped to land on T_end
+  double dt_cfl;                  // cfl / rate of the state after dt_cfl_step steps (0: not known)
+  long long dt_cfl_step;
 };
 
 // Hybrid limiter (Algorithm 1) of one solver: the stage kernel stores the unfiltered DG solution
@@ -188,13 +190,84 @@ __device__ __forceinline__ float arcp(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-__device__ __forceinline__ double arcp(double x) { return 1.0 / x; }
+// FP64: the FP64 pipe issues one warp instruction every 16 cycles, and the library's correctly rounded
+// division and square root take about 8 and 10 of them. From the hardware's 20-bit approximation r one
+// third-order Newton-Householder step gives 1/x = r (1 + e + e^2 + O(e^3)), e = 1 - x r, to about an
+// ulp in 3 instructions.
+__device__ __forceinline__ double arcp(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
 __device__ __forceinline__ float asqrt(float x) {
   float r;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-__device__ __forceinline__ double asqrt(double x) { return sqrt(x); }
+// FP64: from y ~ 1/sqrt(x) (20 bits) and g = x y, sqrt(x) = g (1 - e)^(-1/2) with e = 1 - g y, by the
+// binomial series to second order (the next term is 5/16 e^3): 5 instructions, about an ulp. Zeros,
+// subnormals and negative arguments (NaN) take the library's function.
+__device__ __forceinline__ double asqrt(double x) {
+  if (__double2hiint(x) < 0x00200000) return sqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double g = x * y;
+  const double e = fma(-g, y, 1.0);
+  return fma(g * e, fma(e, 0.375, 0.5), g);
+}
+
+// Bits of |x|; their order is the order of the magnitudes, with NaNs above infinity.
+__device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffll; }
+// 0 < x < infinity, in integer arithmetic (the FP64 pipe takes no part)
+__device__ __forceinline__ bool pos_finite(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b < 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool not_finite(double x) { return abs_bits(x) >= 0x7ff0000000000000ll; }
+__device__ __forceinline__ bool not_finite(float x) { return !isfinite(x); }
+__device__ __forceinline__ bool pos_finite(float x) { return x > 0.f && isfinite(x); }
+
+// Damping factors f[l] = exp(x[l]), l = 1..N-1, of x <= 0 that decreases with l. FP32: 2^(x log2 e) by the
+// hardware's approximate exponential (about 2 ulp; a factor in (0, 1]). FP64: where the solution is
+// smooth the arguments are tiny, and if all of the warp's are, the Taylor polynomial of degree 6
+// (|x| < 2^-9: the next term is below 2^-75) or 10 (|x| < 2^-4: below 2^-69) is exact to rounding in 6 or
+// 10 instructions instead of the function's 15 or more. Called by all lanes of the warp.
+template <int N>
+__device__ __forceinline__ void exp_damp(const float (&x)[N], float (&f)[N]) {
+#pragma unroll
+  for (int l = 1; l < N; ++l) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x[l] * 1.4426950408889634f));
+    f[l] = y;
+  }
+}
+template <int N>
+__device__ __forceinline__ void exp_damp(const double (&x)[N], double (&f)[N]) {
+  const long long big = abs_bits(x[N - 1]);
+  if (!__any_sync(0xffffffffu, big >= 0x3fb0000000000000ll)) {
+    const bool tiny = !__any_sync(0xffffffffu, big >= 0x3f60000000000000ll);
+#pragma unroll
+    for (int l = 1; l < N; ++l) {
+      double p = 1.0 / 720.0;
+      if (!tiny) {
+        p = fma(x[l], 1.0 / 3628800.0, 1.0 / 362880.0);
+        p = fma(x[l], p, 1.0 / 40320.0);
+        p = fma(x[l], p, 1.0 / 5040.0);
+        p = fma(x[l], p, 1.0 / 720.0);
+      }
+      p = fma(x[l], p, 1.0 / 120.0);
+      p = fma(x[l], p, 1.0 / 24.0);
+      p = fma(x[l], p, 1.0 / 6.0);
+      p = fma(x[l], p, 0.5);
+      p = fma(x[l], p, 1.0);
+      f[l] = fma(x[l], p, 1.0);
+    }
+  } else {
+#pragma unroll
+    for (int l = 1; l < N; ++l) f[l] = exp(x[l]);
+  }
+}
 
 // ---- fluxes ------------------------------------------------------------------------------
 // 1D flux of u (NV = 1 or 3).
@@ -285,11 +358,12 @@ __device__ __forceinline__ T speed2d(const T* u, T gamma, T gm1, T ax, T ay) {
   }
 }
 
-// max that keeps a NaN: a non-physical trace (p < 0 gives a NaN sound speed) must reach the cell
-// averages and be reported, not be hidden by the other side's wave speed.
-template <class T>
-__device__ __forceinline__ T nan_max(T a, T b) {
-  return (a > b || a != a) ? a : b;
+// Max of two non-negative values that keeps a NaN: a non-physical trace (p < 0 gives a NaN sound speed)
+// must reach the cell averages and be reported, not be hidden by the other side's wave speed. FP64: on
+// the bits, in integer instructions.
+__device__ __forceinline__ double nan_max(double a, double b) {
+  const long long x = abs_bits(a), y = abs_bits(b);
+  return __longlong_as_double(x > y ? x : y);
 }
 // FP32: the same in one instruction (max.NaN returns NaN if either operand is NaN)
 __device__ __forceinline__ float nan_max(float a, float b) {
@@ -298,16 +372,39 @@ __device__ __forceinline__ float nan_max(float a, float b) {
   return r;
 }
 
-// Local Lax–Friedrichs flux for a 1D face: fh = 1/2 (f(uL) + f(uR)) - 1/2 alpha (uR - uL).
+// Multiply-add and product rounded as written: the compiler fuses a product into either of two sums, and
+// which one may differ from kernel to kernel; with these a cell's result is the same in each.
+__device__ __forceinline__ float tfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double tfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float tmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double tmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float tadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double tadd(double a, double b) { return __dadd_rn(a, b); }
+
+// Local Lax–Friedrichs flux of a face, fh = 1/2 (f(uL) + f(uR)) - 1/2 alpha (uR - uL), alpha the larger
+// spectral radius; in 1D twice it: f(uL) + f(uR) - alpha (uR - uL) (the halving is folded into its uses).
 template <int EQ, class T>
-__device__ __forceinline__ void llf1d(const T* uL, const T* uR, T* fh, T gamma, T gm1, T ax) {
-  constexpr int NV = EQ == EQ_EULER ? 3 : 1;
-  T fL[NV], fR[NV];
-  flux1d<EQ>(uL, fL, gm1, ax);
-  flux1d<EQ>(uR, fR, gm1, ax);
-  T a = nan_max(speed1d<EQ>(uL, gamma, gm1, ax), speed1d<EQ>(uR, gamma, gm1, ax));
-#pragma unroll
-  for (int v = 0; v < NV; ++v) fh[v] = T(0.5) * (fL[v] + fR[v]) - T(0.5) * a * (uR[v] - uL[v]);
+__device__ __forceinline__ void llf1d_twice(const T* uL, const T* uR, T* fh, T gamma, T gm1, T ax) {
+  if constexpr (EQ == EQ_EULER) {
+    const T iL = arcp(uL[0]), iR = arcp(uR[0]);
+    const T vL = tmul(uL[1], iL), vR = tmul(uR[1], iR);
+    const T pL = tmul(gm1, tfma(tmul(T(-0.5), uL[1]), vL, uL[2]));
+    const T pR = tmul(gm1, tfma(tmul(T(-0.5), uR[1]), vR, uR[2]));
+    const T cL = asqrt(tmul(tmul(gamma, pL), iL)), cR = asqrt(tmul(tmul(gamma, pR), iR));
+    const T a = nan_max(tadd(fabs(vL), cL), tadd(fabs(vR), cR));
+    const T s0 = tadd(uL[1], uR[1]);
+    const T s1 = tfma(uL[1], vL, tfma(uR[1], vR, tadd(pL, pR)));
+    const T s2 = tfma(vL, tadd(uL[2], pL), tmul(vR, tadd(uR[2], pR)));
+    fh[0] = tfma(-a, tadd(uR[0], -uL[0]), s0);
+    fh[1] = tfma(-a, tadd(uR[1], -uL[1]), s1);
+    fh[2] = tfma(-a, tadd(uR[2], -uL[2]), s2);
+  } else {
+    T fL[1], fR[1];
+    flux1d<EQ>(uL, fL, gm1, ax);
+    flux1d<EQ>(uR, fR, gm1, ax);
+    const T a = nan_max(speed1d<EQ>(uL, gamma, gm1, ax), speed1d<EQ>(uR, gamma, gm1, ax));
+    fh[0] = (fL[0] + fR[0]) - a * (uR[0] - uL[0]);
+  }
 }
 
 template <int EQ, int DIR, class T>
@@ -321,6 +418,10 @@ __device__ __forceinline__ void llf2d(const T* uL, const T* uR, T* fh, T gamma, 
   for (int v = 0; v < NV; ++v) fh[v] = T(0.5) * (fL[v] + fR[v]) - T(0.5) * a * (uR[v] - uL[v]);
 }
 
+// Max of two non-negative values whose NaNs need not be kept (FP64: they are).
+__device__ __forceinline__ float keep_max(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double keep_max(double a, double b) { return nan_max(a, b); }
+
 // Cell-average quantities for the filter and the CFL rate: beta^x, beta^y, 1/Hbar.
 template <int EQ, int DIM, class T>
 __device__ __forceinline__ void avg_params(const T* ub, T gamma, T gm1, T ax, T ay, T& bx, T& by,
@@ -329,12 +430,12 @@ __device__ __forceinline__ void avg_params(const T* ub, T gamma, T gm1, T ax, T 
     bx = fabs(ax);
     by = fabs(ay);
     invH = T(1);
-    physical = isfinite(ub[0]);
+    physical = !not_finite(ub[0]);
   } else if constexpr (EQ == EQ_BURG) {
     bx = fabs(ub[0]);
     by = bx;
     invH = T(1);
-    physical = isfinite(ub[0]);
+    physical = !not_finite(ub[0]);
   } else if constexpr (DIM == 1) {
     const T inv = arcp(ub[0]);
     T vel = ub[1] * inv;
@@ -343,7 +444,7 @@ __device__ __forceinline__ void avg_params(const T* ub, T gamma, T gm1, T ax, T 
     bx = fabs(vel) + c;
     by = T(0);
     invH = ub[0] * arcp(ub[2] + p);
-    physical = (ub[0] > T(0)) && (p > T(0)) && isfinite(bx) && isfinite(invH);
+    physical = pos_finite(ub[0]) && pos_finite(p) && pos_finite(bx) && pos_finite(invH);
   } else {
     T inv = arcp(ub[0]);
     T vx = ub[1] * inv, vy = ub[2] * inv;
@@ -352,7 +453,7 @@ __device__ __forceinline__ void avg_params(const T* ub, T gamma, T gm1, T ax, T 
     bx = fabs(vx) + c;
     by = fabs(vy) + c;
     invH = ub[0] * arcp(ub[3] + p);
-    physical = (ub[0] > T(0)) && (p > T(0)) && isfinite(bx) && isfinite(by) && isfinite(invH);
+    physical = pos_finite(ub[0]) && pos_finite(p) && pos_finite(bx) && pos_finite(by) && pos_finite(invH);
   }
 }
 
@@ -607,7 +708,7 @@ __device__ __forceinline__ double vabs(double x) { return fabs(x); }
 __device__ __forceinline__ f2 vabs(f2 x) { return f2{fabsf(x.x), fabsf(x.y)}; }
 // max(|a|, |b|), lane by lane
 __device__ __forceinline__ float vmaxabs(float a, float b) { return fmaxf(fabsf(a), fabsf(b)); }
-__device__ __forceinline__ double vmaxabs(double a, double b) { return fmax(fabs(a), fabs(b)); }
+__device__ __forceinline__ double vmaxabs(double a, double b) { return nan_max(a, b); }
 __device__ __forceinline__ f2 vmaxabs(f2 a, f2 b) {
   return f2{fmaxf(fabsf(a.x), fabsf(b.x)), fmaxf(fabsf(a.y), fabsf(b.y))};
 }

@@ -29,6 +29,13 @@ int default_block_warps(const StageLauncher& L, int max_wpb);
 
 // Instantiation tables (one per kernel file). Return {nullptr} if the combination is not compiled.
 StageLauncher stage1d_launcher(int K, int EQ, int PREC, bool oedg = false);
+// The 1D kernel of a whole step, and its threads, blocks and tiles for n cells.
+StageLauncher step1d_launcher(int K, int EQ, int PREC);
+struct Step1DGrid {
+  unsigned block, grid;
+  long long tiles;
+};
+Step1DGrid step1d_grid(const StageLauncher& L, long long n);
 StageLauncher stage2d_f64_launcher(int K, int EQ, int BASIS);
 StageLauncher stage2d_f32_launcher(int K, int EQ, int BASIS);
 StageLauncher stage2d_oedg_launcher(int K, int EQ, int BASIS, int PREC);  // OEDG form: Burgers, Euler

@@ -51,6 +51,8 @@ __global__ void noalloc_reset(DevScalars* sc) {
     sc->err = 0u;
     sc->blocks_done = 0u;
     sc->is_last = 0u;
+    sc->dt_cfl = 0.0;
+    sc->dt_cfl_step = 0;
   }
 }
 
@@ -95,38 +97,33 @@ extern "C" dg_status dg_step_noalloc(const dg_mesh* m, int k, int eq, const dg_f
   if (cudaGetLastError() != cudaSuccess) return DG_ERR_CUDA;
   if (launch_rate(g, u_in, sc, 0, st) != cudaSuccess) return DG_ERR_CUDA;
 
-  static const double C0[3] = {0.0, 0.75, 1.0 / 3.0};
-  static const double C1[3] = {1.0, 0.25, 2.0 / 3.0};
   const void* srcs[3] = {u_in, b1, b2};
   void* dsts[3] = {b1, b2, u_out};
   if (dim == 1) {
-    StageLauncher L = stage1d_launcher(k, eq, PREC_F64);
+    const StageLauncher L = step1d_launcher(k, eq, PREC_F64);   // the whole step: no stage states
     if (!L.launch) return DG_ERR_UNSUPPORTED;
-    const int nwarps = (m->nx + STRIP_OUT - 1) / STRIP_OUT;
-    for (int s = 0; s < 3; ++s) {
-      Stage1DArgs a;
-      a.uin = srcs[s];
-      a.un = u_in;
-      a.uout = dsts[s];
-      a.nx = m->nx;
-      a.ncell = ncell;
-      a.h = g.hx;
-      a.bc = m->bc[0];
-      a.c0 = C0[s];
-      a.c1 = C1[s];
-      a.stage = s;
-      a.filter_on = p->enabled ? FILT_JUMP + p->filter_kind : FILT_OFF;
-      a.gamma = p->gamma;
-      a.ax = p->adv_speed[0];
-      a.cfl = p->cfl;
-      a.nwarps = nwarps;
-      a.positivity = (p->positivity && eq == DG_EQ_EULER) ? 1 : 0;
-      a.hybrid = 0;
-      a.hyb = HybridOut{};
-      a.sc = sc;
-      stage1d_consts(a);
-      if (L.launch(&a, (unsigned)((nwarps + 3) / 4), 128, 256, st) != cudaSuccess) return DG_ERR_CUDA;
-    }
+    const Step1DGrid sg = step1d_grid(L, m->nx);
+    Stage1DArgs a;
+    a.uin = a.un = u_in;
+    a.uout = u_out;
+    a.nx = m->nx;
+    a.ncell = ncell;
+    a.h = g.hx;
+    a.bc = m->bc[0];
+    a.c0 = 0.0;
+    a.c1 = 1.0;
+    a.stage = 0;
+    a.filter_on = p->enabled ? FILT_JUMP + p->filter_kind : FILT_OFF;
+    a.gamma = p->gamma;
+    a.ax = p->adv_speed[0];
+    a.cfl = p->cfl;
+    a.nwarps = sg.tiles;
+    a.positivity = (p->positivity && eq == DG_EQ_EULER) ? 1 : 0;
+    a.hybrid = 0;
+    a.hyb = HybridOut{};
+    a.sc = sc;
+    stage1d_consts(a);
+    if (L.launch(&a, sg.grid, sg.block, 0, st) != cudaSuccess) return DG_ERR_CUDA;
   } else {
     StageLauncher L = stage2d_f64_launcher(k, eq, basis);
     if (!L.launch) return DG_ERR_UNSUPPORTED;
@@ -153,8 +150,8 @@ extern "C" dg_status dg_step_noalloc(const dg_mesh* m, int k, int eq, const dg_f
       a.hy = g.hy;
       a.bcx = m->bc[0];
       a.bcy = m->bc[2];
-      a.c0 = C0[s];
-      a.c1 = C1[s];
+      a.c0 = so_c0(s);
+      a.c1 = so_c1(s);
       a.stage = s;
       a.filter_on = p->enabled ? FILT_JUMP + p->filter_kind : FILT_OFF;
       a.gamma = p->gamma;

@@ -29,6 +29,8 @@ struct dg_solver {
   unsigned grid, block;
   size_t smem;
   int nstrips, nchunks, nwarps1d;
+  bool whole_step;          // 1D: one launch per step (step1d_kernel) instead of one per stage
+  long long ntiles1d;       // its tiles
   cudaGraphExec_t pair_exec;
   bool pair_ready;
   long long pair_launches;  // kernel nodes in the step-pair graph

@@ -1412,21 +1412,10 @@ struct Stage2D {
             }
           } else if (a.filter_on) {
             T fac[LMAX + 1];
-            if constexpr (PR::MIXED) {
-              // exp(-sigma dt) as 2^(-sigma dt log2 e) by the hardware's approximate exponential
-              // (about 2 ulp; a damping factor in (0, 1])
-              const T dtl = dt * T(1.4426950408889634);
+            const T damp = -(invH2 * dt);
 #pragma unroll
-              for (int l = 1; l <= LMAX; ++l) {
-                const float x = -(sig[l] * invH2) * dtl;
-                float f;
-                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(x));
-                fac[l] = f;
-              }
-            } else {
-#pragma unroll
-              for (int l = 1; l <= LMAX; ++l) fac[l] = exp(-(sig[l] * invH2) * dt);
-            }
+            for (int l = 1; l <= LMAX; ++l) sig[l] *= damp;
+            exp_damp(sig, fac);
             if (a.filter_on == FILT_GLOBAL) {
               // one coefficient for every mode, from the jumps of all derivative orders (Eq. para:damp)
 #pragma unroll
@@ -1635,7 +1624,7 @@ struct Stage2D {
         }
         __syncwarp();
         T th1 = T(1), th2 = T(1);
-        limit_cells(mask, ws, slot, eps_r, eps, rmin, gam, gm1, ihx, ihy, th1, th2, rate);
+        limit_cells(mask, ws, slot, eps_r, eps, gam, gm1, ihx, ihy, th1, th2, rate);
         if (fails) {
           const T th = th1 * th2;
 #pragma unroll
@@ -1669,7 +1658,7 @@ struct Stage2D {
   // theta_1, theta_2 and the limited cell's rate for the cells of the lanes in mask, which hold their
   // coefficients in row slot `slot`: lane i evaluates point i (and i + 32) of each cell and solves for
   // its own largest admissible theta_2. Rolled, so that the rare path costs the others no registers.
-  static __device__ __noinline__ void limit_cells(unsigned mask, T* ws, int slot, T eps_r_, T eps_, T rmin_, T gam,
+  static __device__ __noinline__ void limit_cells(unsigned mask, T* ws, int slot, T eps_r_, T eps_, T gam,
                                                   T gm1, T ihx, T ihy, T& th1_, T& th2_, T& rate_) {
     constexpr int PER = (NP_LIM + 31) / 32;
     const int lane = threadIdx.x & 31;
@@ -1686,7 +1675,6 @@ struct Stage2D {
       const int j = __ffs(mask) - 1;
       mask &= mask - 1;
       const T eps_r = __shfl_sync(0xffffffffu, eps_r_, j), eps = __shfl_sync(0xffffffffu, eps_, j);
-      const T rmin = __shfl_sync(0xffffffffu, rmin_, j);
       T ub[NV], w[PER][NV], th1 = T(1), th2 = T(1);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
@@ -1700,10 +1688,18 @@ struct Stage2D {
           for (int i = 0; i < PER; ++i) w[i][v] += c[i][m] * x;
         }
       }
-      if (rmin < eps_r) th1 = (ub[0] - eps_r) / (ub[0] - rmin);
+      // density: rho_bar + theta_1 (rho - rho_bar) = eps_r + theta_1 (rho - rho_min), which keeps the digits
+      // of a density far below the average
+      T low = w[0][0];
+#pragma unroll
+      for (int i = 1; i < PER; ++i) low = fmin(low, w[i][0]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) low = fmin(low, __shfl_xor_sync(0xffffffffu, low, o));
+      const bool thin = low < eps_r;
+      if (thin) th1 = (ub[0] - eps_r) / (ub[0] - low);
 #pragma unroll
       for (int i = 0; i < PER; ++i) {
-        w[i][0] = ub[0] + th1 * (w[i][0] - ub[0]);
+        if (thin) w[i][0] = eps_r + th1 * (w[i][0] - low);
         if (pressure_of<NV>(w[i], gm1) < eps) th2 = pp_segment<NV>(ub, w[i], eps, gm1, th2);
       }
 #pragma unroll
@@ -1737,7 +1733,7 @@ struct Stage2D {
       if (blockIdx.x == 0 && threadIdx.x == 0) a.oe.sc->active = 1u;
     }
     const int wib = threadIdx.x >> 5;
-    double* red = (double*)smem;                                  // 32 doubles for stage_end
+    T* red = (T*)smem;                                            // 32 words for stage_end
     T* ws = (T*)(smem + 256 + warp_bytes() * wib);
     const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + wib;
     double my_rate = 0.0;
@@ -1745,8 +1741,8 @@ struct Stage2D {
     bool my_ok = true;
     if (gw < (long long)a.nstrips * a.nchunks)
       item(a, ctl.dt, (int)(gw % a.nstrips), (int)(gw / a.nstrips), ws, my_rate, my_rate_t, my_ok);
-    if constexpr (PR::MIXED) my_rate = (double)my_rate_t;
-    stage_end(a.sc, a.stage, my_rate, my_ok, red);
+    if constexpr (PR::MIXED) stage_end(a.sc, a.stage, ctl, a.cfl, my_rate_t, 1.0, my_ok, red);
+    else stage_end(a.sc, a.stage, ctl, a.cfl, my_rate, 1.0, my_ok, red);
   }
 };
 

@@ -11,10 +11,14 @@
 //
 // Protocol on DevScalars (no spin-waits anywhere):
 //   - every stage kernel returns at once if done or err is set (values fixed during the launch);
-//   - stage 0: all threads compute the same dt from (t, T_end, rate_bits[step & 1]); block 0
-//     publishes dt and is_last, clears rate_bits[(step + 1) & 1] and the last-block counter;
+//   - stage 0: every block takes the same dt from (t, T_end) and cfl / rate, which the last block of
+//     the previous step left in dt_cfl (the first step divides by rate_bits[step & 1] itself); block 0
+//     publishes dt and is_last;
 //   - stage 2: every block atomically maxes its rate into rate_bits[(step + 1) & 1], then counts
-//     itself done; the last block (threadfence reduction) advances t and step, and sets done.
+//     itself done; the last block (threadfence reduction) advances t and step, sets done, and clears
+//     the counter and the slot that the next step will max into. So between steps the counter and
+//     rate_bits[(step + 1) & 1] are zero whoever made the last step, and a kernel that runs all three
+//     stages needs no block to clear them while others may already have finished.
 #pragma once
 #include "dg_device.cuh"
 
@@ -111,79 +115,89 @@ struct Tab2D {
 struct StageCtl {
   bool run;
   double dt;
+  long long step;
 };
 
-__device__ __forceinline__ StageCtl stage_begin(DevScalars* sc, int stage, double cfl) {
-  volatile DevScalars* vs = sc;
-  StageCtl c{false, 0.0};
-  if (vs->done | vs->err) return c;
-  if (stage == 0) {
-    long long step = vs->step;
-    double rate = __longlong_as_double((long long)vs->rate_bits[step & 1]);
-    if (!(rate > 0.0) || !isfinite(rate)) {
-      if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) atomicOr(&sc->err, ERRB_RATE);
-      return c;
-    }
-    double t = vs->t, T = vs->T_end;
-    double dtc = cfl / rate;
-    bool last = (t + dtc >= T);
-    c.dt = last ? T - t : dtc;
-    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) {
-      sc->dt = c.dt;
-      sc->is_last = last ? 1u : 0u;
-      sc->rate_bits[(step + 1) & 1] = 0ull;
-      sc->blocks_done = 0u;
-    }
-  } else {
-    c.dt = vs->dt;
-  }
-  c.run = true;
-  return c;
+// The unclipped step size of the step after `step` completed ones, 0 if the rate gives none.
+__device__ __forceinline__ double cfl_step(const DevScalars* sc, long long step, double cfl) {
+  const double rate = __longlong_as_double((long long)((volatile const DevScalars*)sc)->rate_bits[step & 1]);
+  return (rate > 0.0) && isfinite(rate) ? cfl / rate : 0.0;
 }
 
-// Block-level end of a stage: publish non-physical flags; in the final stage also the rate max
-// and the last-block step advance. Every thread of the block must call it (uses __syncthreads).
-__device__ __forceinline__ void stage_end(DevScalars* sc, int stage, double my_rate, bool my_ok,
-                                          double* red_buf /* >= 32 doubles of shared memory */) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  double r = warp_max(my_rate);
-  unsigned bad = __ballot_sync(0xffffffffu, !my_ok);
-  __shared__ unsigned s_bad;
-  __shared__ bool s_last;
-  if (threadIdx.x == 0) s_bad = 0u;
-  __syncthreads();
-  if (lane == 0) {
-    red_buf[wid] = r;
-    if (bad) atomicOr(&s_bad, 1u);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = 0.0;
-    for (int w = 0; w < nw; ++w) m = (red_buf[w] > m || red_buf[w] != red_buf[w]) ? red_buf[w] : m;
-    if (s_bad) atomicOr(&sc->err, ERRB_NONPHYS);
-    s_last = false;
-    if (stage == 2) {
-      long long step = ((volatile DevScalars*)sc)->step;
-      atomic_max_nonneg(&sc->rate_bits[(step + 1) & 1], m);
-      __threadfence();
-      unsigned nblocks = gridDim.x * gridDim.y;
-      unsigned prev = atomicAdd(&sc->blocks_done, 1u);
-      s_last = (prev == nblocks - 1);
-    }
-  }
-  __syncthreads();
-  if (stage == 2 && s_last && threadIdx.x == 0) {
-    __threadfence();
+// Block-level begin of a stage, called by every thread (uses __syncthreads). The scalars are read and
+// the step size formed by warp 0 alone: an FP64 warp instruction holds its quarter of the SM for 64
+// cycles, so the same few operations in every warp cost a 15-warp SM 6000 cycles, as much as two stages
+// of a 1D solve. extra(lane, ctl) runs in warp 0 before the barrier, for the block's own constants.
+template <class F>
+__device__ __forceinline__ StageCtl stage_begin(DevScalars* sc, int stage, double cfl, F&& extra) {
+  __shared__ StageCtl s_ctl;
+  if (threadIdx.x < 32) {
+    const bool first = threadIdx.x == 0 && blockIdx.x == 0;
     volatile DevScalars* vs = sc;
-    if (vs->err == 0u) {
-      double t = vs->t;
-      double tn = vs->is_last ? vs->T_end : t + vs->dt;
-      long long st = vs->step + 1;
-      vs->t = tn;
-      vs->step = st;
-      vs->done = (tn >= vs->T_end || st >= vs->max_step) ? 1u : 0u;
+    const unsigned done = vs->done, err = vs->err;
+    const long long step = vs->step, at = vs->dt_cfl_step;
+    const double t = vs->t, T = vs->T_end, pub = vs->dt;
+    double dtc = vs->dt_cfl;
+    StageCtl c{(done | err) == 0u, pub, step};
+    if (stage == 0 && c.run) {
+      if (!(at == step && dtc > 0.0)) dtc = cfl_step(sc, step, cfl);
+      if (dtc > 0.0) {
+        const bool last = (t + dtc >= T);
+        c.dt = last ? T - t : dtc;
+        if (first) {
+          sc->dt = c.dt;
+          sc->is_last = last ? 1u : 0u;
+        }
+      } else {
+        c.run = false;
+        if (first) atomicOr(&sc->err, ERRB_RATE);
+      }
     }
+    if (c.run) extra((int)threadIdx.x, c);
+    if (threadIdx.x == 0) s_ctl = c;
   }
+  __syncthreads();
+  return s_ctl;
+}
+__device__ __forceinline__ StageCtl stage_begin(DevScalars* sc, int stage, double cfl) {
+  return stage_begin(sc, stage, cfl, [](int, const StageCtl&) {});
+}
+
+// Block-level end of a stage: publish non-physical flags; in the final stage also the rate max (my_rate
+// times `scale`, reduced in the stage's own arithmetic, scaled in FP64) and the last-block step advance.
+// Every thread of the block must call it (uses __syncthreads).
+template <class T>
+__device__ __forceinline__ void stage_end(DevScalars* sc, int stage, const StageCtl& ctl, double cfl, T my_rate,
+                                          double scale, bool my_ok, T* red /* >= 32 words of shared memory */) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  T r = my_rate;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) r = nan_max(__shfl_xor_sync(0xffffffffu, r, o), r);
+  if (lane == 0) red[wid] = r;
+  const bool bad = __syncthreads_or(!my_ok) != 0;
+  if (threadIdx.x != 0) return;
+  if (bad) atomicOr(&sc->err, ERRB_NONPHYS);
+  if (stage != 2) return;
+  for (int w = 1; w < nw; ++w) r = nan_max(red[w], r);
+  const long long st = ctl.step + 1;
+  atomic_max_nonneg(&sc->rate_bits[st & 1], (double)r * scale);
+  __threadfence();
+  if (atomicAdd(&sc->blocks_done, 1u) != gridDim.x * gridDim.y - 1) return;
+  __threadfence();
+  volatile DevScalars* vs = sc;
+  const unsigned err = vs->err, last = vs->is_last;
+  const double t = vs->t, T_end = vs->T_end;
+  const long long max_step = vs->max_step;
+  if (err == 0u) {
+    const double tn = last ? T_end : t + ctl.dt;
+    vs->t = tn;
+    vs->step = st;
+    vs->done = (tn >= T_end || st >= max_step) ? 1u : 0u;
+    vs->rate_bits[(st + 1) & 1] = 0ull;
+    vs->dt_cfl = cfl_step(sc, st, cfl);
+    vs->dt_cfl_step = st;
+  }
+  vs->blocks_done = 0u;
 }
 
 // Hybrid limiter (Algorithm 1), one row of output cells of a warp: eta and the filter factors of the
