@@ -209,50 +209,62 @@ extern "C" dg_status dg_workspace_size(const dg_mesh* mesh, int degree, int equa
   return DG_OK;
 }
 
-// One warp per (strip, chunk) item, so a 2D stage launch runs in waves of the resident warps. A
-// warp sweeps H + 4 rows (two halo rows on each side): pick the H that minimises waves x (H + 4),
-// never below 8 rows (the halo would dominate).
-int dgk::default_chunk_rows(const StageLauncher& L, int nstrips, int ny, int wpb, unsigned block, size_t smem) {
+int dgk::device_sms() {
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0)
     nsm = 152;
-  int bps = L.blocks_per_sm ? L.blocks_per_sm(block, smem) : 0;
-  if (bps <= 0) bps = 1;
-  const long long W = (long long)nsm * bps * wpb;
-  long long best = -1;
-  int H = 8;
-  for (int w = 1; w <= 16; ++w) {
-    long long nch = w * W / nstrips;
-    if (nch < 1) nch = 1;
-    if (nch > ny) nch = ny;
-    int h = (int)((ny + nch - 1) / nch);
-    if (h < 8) h = 8;
-    const long long items = (long long)nstrips * ((ny + h - 1) / h);
-    const long long cost = ((items + W - 1) / W) * (h + 4);
-    if (best < 0 || cost < best) {
-      best = cost;
-      H = h;
-    }
-  }
-  return H;
+  return nsm;
 }
 
-// Warps per block when the caller gives none: of 4, 2, 8 and 1 warps (within max_wpb, the row-slot
-// limit), the block with the most resident warps per SM; ties keep the earlier candidate.
-int dgk::default_block_warps(const StageLauncher& L, int max_wpb) {
-  int best = -1, wpb = max_wpb < 4 ? max_wpb : 4;
-  for (int c : {4, 2, 8, 1}) {
-    if (c > max_wpb) continue;
-    const size_t smem = 256 + L.slot_bytes_per_warp * c;
+// A 2D stage launch runs one warp per (strip, chunk) item; a warp sweeps its rows and the halo rows, which
+// cost about three rows' work in the FP32 form and two in FP64 (their guarded parts are skipped). What
+// a row costs depends on the warps that share the SM. FP32 form: a quarter of an SM that holds one warp
+// runs at its latency, two take 1.5 times as long (2048^2 Q2: 5400 and 4030 cycles per row and warp).
+// FP64: the pipe serves the whole SM, and four warps fill it. More warps than are resident run in
+// rounds. So few rows per chunk where the mesh leaves quarters idle, and many where it fills them.
+double dgk::tile_cost(long long items, int rows, int warps, int resident, int nsm, bool fp64) {
+  const long long blocks = (items + warps - 1) / warps;
+  const long long w = ((blocks + nsm - 1) / nsm) * warps;
+  auto shared = [&](long long n) -> double {
+    if (n <= 0) return 0.0;
+    return fp64 ? (n > 4 ? 0.25 * n : 1.0) : 0.5 + 0.5 * (double)((n + 3) / 4);
+  };
+  return ((double)(w / resident) * shared(resident) + shared(w % resident)) * (rows + (fp64 ? 2 : 3));
+}
+
+// Per step, with the rule before (the fewest waves of the largest blocks, never below 8 rows) and this
+// one: Q2 FP32 form 64^2 102 -> 46 us, 128^2 102 -> 55, 256^2 104 -> 83, with the limiter 128^2 122 -> 60;
+// Q3 128^2 280 -> 122; FP64 Q2 128^2 2225 -> 856, P3 160^2 3046 -> 1318; from 512^2 on the same.
+TileShape dgk::tile_shape(const StageLauncher& L, int nstrips, int ny, bool fp64, int rows, int warps) {
+  // at most the row slots that fit in 200 KB of shared memory
+  int most = (int)((200 * 1024 - 256) / L.slot_bytes_per_warp);
+  if (most > 8) most = 8;
+  if (most < 1) return TileShape{0, 0};
+  const int nsm = device_sms();
+  TileShape best{0, 0};
+  double cost = -1.0;
+  for (int c : {4, 2, 1, 8}) {
+    if (warps > 0 ? c != 4 : c > most) continue;
+    const int wpb = warps > 0 ? (warps < most ? warps : most) : c;
+    const size_t smem = 256 + L.slot_bytes_per_warp * wpb;
     if (L.set_smem(smem) != cudaSuccess) continue;
-    const int bps = L.blocks_per_sm ? L.blocks_per_sm(32u * c, smem) : 0;
-    if (bps * c > best) {
-      best = bps * c;
-      wpb = c;
+    const int bps = L.blocks_per_sm ? L.blocks_per_sm(32u * wpb, smem) : 0;
+    if (bps < 1) continue;
+    for (int w = 1; w <= 64; ++w) {                     // warps per SM
+      long long nch = (long long)w * nsm / nstrips;
+      nch = nch < 1 ? 1 : (nch > ny ? ny : nch);
+      const int H = rows > 0 ? (rows < ny ? rows : ny) : (int)((ny + nch - 1) / nch);
+      const double t = tile_cost((long long)nstrips * ((ny + H - 1) / H), H, wpb, bps * wpb, nsm, fp64);
+      if (cost < 0.0 || t < cost) {
+        cost = t;
+        best = TileShape{H, wpb};
+      }
+      if (rows > 0 || nch == ny) break;
     }
   }
-  return wpb;
+  if (best.warps > 0 && L.set_smem(256 + L.slot_bytes_per_warp * best.warps) != cudaSuccess) return TileShape{0, 0};
+  return best;
 }
 
 static dg_status setup_launch(dg_solver* s, int tile_rows, int tile_warps) {
@@ -289,23 +301,13 @@ static dg_status setup_launch(dg_solver* s, int tile_rows, int tile_warps) {
   if (!s->L.launch) return DG_ERR_UNSUPPORTED;
   const int nx = s->mesh.nx, ny = s->mesh.ny;
   s->nstrips = (nx + STRIP_OUT - 1) / STRIP_OUT;
-  // warps per block: the caller's, else the block size with the most resident warps; at most the
-  // row slots that fit in 200 KB of shared memory
-  size_t per_warp = s->L.slot_bytes_per_warp;
-  int wpb = (int)((200 * 1024 - 256) / per_warp);
-  if (wpb > 8) wpb = 8;
-  if (wpb < 1) return DG_ERR_UNSUPPORTED;
-  if (tile_warps > 0) {
-    if (tile_warps < wpb) wpb = tile_warps;
-  } else {
-    wpb = default_block_warps(s->L, wpb);
-  }
+  const TileShape tile = tile_shape(s->L, s->nstrips, ny, s->prec == PREC_F64, tile_rows, tile_warps);
+  if (tile.warps < 1) return DG_ERR_UNSUPPORTED;
+  const int wpb = tile.warps, H = tile.rows;
+  s->own_tile = tile_rows <= 0;
   s->warps_per_block = wpb;
   s->block = 32 * wpb;
-  s->smem = 256 + per_warp * wpb;
-  CK(s->L.set_smem(s->smem));
-  int H = tile_rows > 0 ? tile_rows : default_chunk_rows(s->L, s->nstrips, ny, wpb, s->block, s->smem);
-  if (H > ny) H = ny;
+  s->smem = 256 + s->L.slot_bytes_per_warp * wpb;
   s->H = H;
   s->nchunks = (ny + H - 1) / H;
   long long nw = (long long)s->nstrips * s->nchunks;

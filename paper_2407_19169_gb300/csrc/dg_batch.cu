@@ -610,7 +610,9 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
   // 5 + K (the 2D kernel instantiation a solve runs alone)
   constexpr int NCLS = 9;
   std::vector<BatchInst> host;
+  std::vector<char> own_tile;
   host.reserve(n);
+  own_tile.reserve(n);
   int cls_begin[NCLS], cls_count[NCLS], cls_wpb[NCLS];
   long long cls_items[NCLS];
   for (int c = 0; c < NCLS; ++c) {
@@ -626,7 +628,6 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       for (int b = 0; b < 3; ++b) I.buf[b] = s->buf[b];
       I.sc = s->sc;
       I.ncell = s->geom.ncell;
-      I.item0 = cls_items[c];
       I.nx = s->mesh.nx;
       I.ny = s->dim == 2 ? s->mesh.ny : 1;
       I.bcx = s->mesh.bc[0];
@@ -661,11 +662,10 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
         I.inv_h_d = t.inv_h_d;
         I.inv_h_f = t.inv_h_f;
       }
-      cls_items[c] += (long long)I.nstrips * I.nchunks;
       host.push_back(I);
+      own_tile.push_back(s->dim == 2 && s->own_tile);
     }
     cls_count[c] = (int)host.size() - cls_begin[c];
-    cls_wpb[c] = 4;
   }
 
   dg_status status = DG_OK;
@@ -675,23 +675,17 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
   cudaEvent_t fork = nullptr, join[NCLS] = {};
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
-  cudaError_t e = cudaMalloc(&dinst, sizeof(BatchInst) * host.size());
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(dinst, host.data(), sizeof(BatchInst) * host.size(), cudaMemcpyHostToDevice, main);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
-  for (int c = 0; c < NCLS && e == cudaSuccess; ++c) {
-    e = cudaStreamCreateWithFlags(&side[c], cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[c], cudaEventDisableTiming);
-  }
   // 2D classes: the block size with the most resident warps per SM (the row slots of 4, 2, 8 or 1
   // warps within 200 KB of shared memory) and one wave of resident blocks, whose warps then take
   // contiguous item ranges (measured on GB300, 512 uneven instances: 5.9e10 DOF-stage/s against
   // 4.6e10 with the instances' own 4-warp blocks and 4 blocks per SM). 1D classes: 4 blocks of 4
-  // warps per SM.
+  // warps per SM. The rows per chunk of the instances whose solver has the library's tile are chosen
+  // for the class as a whole: the chunk that is best for a small mesh alone would spend the GPU that the
+  // batch fills on halo rows.
   BatchLauncher BL[NCLS];
   long long cls_cap[NCLS];
-  int nsm = 152;
-  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev0) != cudaSuccess || nsm <= 0) nsm = 152;
+  const int nsm = device_sms();
+  cudaError_t e = cudaSuccess;
   for (int c = 0; c < NCLS && e == cudaSuccess; ++c) {
     BL[c] = batch_launcher(c < 3 ? 1 : 2, c % 3 + 1, c >= 6);
     cls_cap[c] = (long long)nsm * 4;
@@ -711,8 +705,41 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       }
       cls_wpb[c] = bw;
       cls_cap[c] = (long long)nsm * (bb > 0 ? bb : 1);
+      BatchInst* I = host.data() + cls_begin[c];
+      const char* own = own_tile.data() + cls_begin[c];
+      double cost = -1.0;
+      int rows = 8;
+      for (int h : {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64, 96, 128}) {
+        long long items = 0;
+        for (int i = 0; i < cls_count[c]; ++i) {
+          const int hi = own[i] ? (h < I[i].ny ? h : I[i].ny) : I[i].H;
+          items += (long long)I[i].nstrips * ((I[i].ny + hi - 1) / hi);
+        }
+        const double t = tile_cost(items, h, bw, best > 0 ? best : 1, nsm, false);
+        if (cost < 0.0 || t < cost) {
+          cost = t;
+          rows = h;
+        }
+      }
+      for (int i = 0; i < cls_count[c]; ++i) {
+        if (!own[i]) continue;
+        I[i].H = rows < I[i].ny ? rows : I[i].ny;
+        I[i].nchunks = (I[i].ny + I[i].H - 1) / I[i].H;
+      }
+    }
+    for (int i = cls_begin[c]; i < cls_begin[c] + cls_count[c]; ++i) {
+      host[i].item0 = cls_items[c];
+      cls_items[c] += (long long)host[i].nstrips * host[i].nchunks;
     }
     if (cls_count[c] > 0 && BL[c].set_smem) e = BL[c].set_smem(BL[c].warp_bytes * cls_wpb[c]);
+  }
+  if (e == cudaSuccess) e = cudaMalloc(&dinst, sizeof(BatchInst) * host.size());
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(dinst, host.data(), sizeof(BatchInst) * host.size(), cudaMemcpyHostToDevice, main);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+  for (int c = 0; c < NCLS && e == cudaSuccess; ++c) {
+    e = cudaStreamCreateWithFlags(&side[c], cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[c], cudaEventDisableTiming);
   }
   unsigned char* pscr = nullptr;
   bool timed_out = false;

@@ -465,54 +465,66 @@ __device__ __forceinline__ T pressure_of(const T* w, T gm1) {
   else return gm1 * (w[3] - T(0.5) * (w[1] * w[1] + w[2] * w[2]) / w[0]);
 }
 
-// Largest t in [0, top] with p(ub + t (w - ub)) >= eps; top if the pressure holds there. Pressure is a
-// concave function of the conservative state, so on the segment p - eps changes sign once (p(ub) >=
-// eps) and Newton's iteration from a failing point comes down to the root from the right without
-// passing it, quadratically (4 to 6 evaluations instead of the 30 (FP32) and 60 (FP64) of a bisection).
-// Rounding leaves it a few units in the last place on the failing side: from there t steps back, twice
-// as far each time, to the first point where the pressure holds. Both loops are bounded; t = 0 (the
-// average itself) always holds.
-template <int NV, class T>
-__device__ __forceinline__ T pp_segment(const T (&ub)[NV], const T (&w)[NV], T eps, T gm1, T top) {
-  T d[NV];
+// Largest t in [0, 1] with p(ub + t (w - ub)) >= eps, for p(ub) >= eps > p(w). Pressure is a concave
+// function of the conservative state, so on the segment p - eps changes sign once.
+// FP32: bisection (30 halvings).
+template <int NV>
+__device__ __forceinline__ float pp_segment(const float (&ub)[NV], const float (&w)[NV], float eps, float gm1) {
+  float lo = 0.f, hi = 1.f;
+#pragma unroll 1
+  for (int it = 0; it < 30; ++it) {
+    const float mid = 0.5f * (lo + hi);
+    float x[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) x[v] = ub[v] + mid * (w[v] - ub[v]);
+    if (pressure_of<NV>(x, gm1) >= eps) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+// FP64, where an operation costs 64 cycles of the pipe and a bisection 60 evaluations: by the concavity
+// Newton's iteration from the failing point comes down to the root from the right without passing it,
+// quadratically (4 to 6 evaluations). Rounding leaves it a few units in the last place on the failing
+// side: from there t steps back, twice as far each time, to the first point where the pressure holds.
+// Both loops are bounded; t = 0 (the average itself) always holds.
+template <int NV>
+__device__ __forceinline__ double pp_segment(const double (&ub)[NV], const double (&w)[NV], double eps, double gm1) {
+  double d[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) d[v] = w[v] - ub[v];
   // p - eps at t, and its derivative
-  auto gap = [&](T t, T& slope) -> T {
-    T x[NV];
+  auto gap = [&](double t, double& slope) -> double {
+    double x[NV], mm = 0.0, md = 0.0;
 #pragma unroll
     for (int v = 0; v < NV; ++v) x[v] = ub[v] + t * d[v];
-    T mm = T(0), md = T(0);
 #pragma unroll
     for (int v = 1; v < NV - 1; ++v) {
       mm += x[v] * x[v];
       md += x[v] * d[v];
     }
-    const T inv = T(1) / x[0];
-    slope = gm1 * (d[NV - 1] - (md - T(0.5) * mm * inv * d[0]) * inv);
-    return gm1 * (x[NV - 1] - T(0.5) * mm / x[0]) - eps;
+    const double inv = 1.0 / x[0];
+    slope = gm1 * (d[NV - 1] - (md - 0.5 * mm * inv * d[0]) * inv);
+    return gm1 * (x[NV - 1] - 0.5 * mm / x[0]) - eps;
   };
-  T t = top, slope;
-  T g = gap(t, slope);
-  const int iters = sizeof(T) == 8 ? 60 : 30;
-  const T ulp = sizeof(T) == 8 ? T(2.3e-16) : T(1.2e-7);
+  const double ulp = 2.3e-16;
+  double t = 1.0, slope;
+  double g = gap(t, slope);
 #pragma unroll 1
-  for (int it = 0; it < iters && g < T(0); ++it) {
-    const T next = t - g / slope;
-    if (!(next < t * (T(1) - ulp)) || !(next > T(0))) break;   // converged, or no descent
+  for (int it = 0; it < 60 && g < 0.0; ++it) {
+    const double next = t - g / slope;
+    if (!(next < t * (1.0 - ulp)) || !(next > 0.0)) break;   // converged, or no descent
     t = next;
     g = gap(t, slope);
   }
-  T back = ulp;
-  const T from = t;
+  const double from = t;
+  double back = ulp;
 #pragma unroll 1
-  for (int it = 0; it < iters && g < T(0); ++it) {
-    t = from * (T(1) - back);
-    if (!(t > T(0))) return T(0);
+  for (int it = 0; it < 60 && g < 0.0; ++it) {
+    t = from * (1.0 - back);
+    if (!(t > 0.0)) return 0.0;
     back += back;
     g = gap(t, slope);
   }
-  return g < T(0) ? T(0) : t;
+  return g < 0.0 ? 0.0 : t;
 }
 
 // ---- storage of the FP32 form ---------------------------------------------------------------

@@ -20,12 +20,17 @@ struct StageLauncher {
   int (*blocks_per_sm)(unsigned block, size_t smem);
 };
 
-// Rows per chunk of the 2D stage kernel when the caller gives none: the fewest waves of resident
-// warps times the rows a warp sweeps (H + 4 halo rows). Queries the current device.
-int default_chunk_rows(const StageLauncher& L, int nstrips, int ny, int wpb, unsigned block, size_t smem);
-// Warps per block of the 2D stage kernel when the caller gives none: the most resident warps per SM
-// (4, 2, 8 or 1 warps, at most max_wpb). Changes the kernel's dynamic shared-memory limit.
-int default_block_warps(const StageLauncher& L, int max_wpb);
+// Tile of the 2D stage kernel: rows per chunk and warps per block (tile_shape in dg_api.cu).
+struct TileShape {
+  int rows, warps;
+};
+// Estimated time of `items` warp items of `rows` rows on nsm SMs that hold `resident` warps each, in
+// blocks of `warps`; in units of one warp's time per row.
+double tile_cost(long long items, int rows, int warps, int resident, int nsm, bool fp64);
+int device_sms();   // SMs of the current device
+// The cheapest tile; rows, warps > 0: the caller's choice of either. {0, 0} if no block fits. Changes the
+// kernel's dynamic shared-memory limit.
+TileShape tile_shape(const StageLauncher& L, int nstrips, int ny, bool fp64, int rows, int warps);
 
 // Instantiation tables (one per kernel file). Return {nullptr} if the combination is not compiled.
 StageLauncher stage1d_launcher(int K, int EQ, int PREC, bool oedg = false);

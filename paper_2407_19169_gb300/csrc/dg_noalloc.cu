@@ -128,14 +128,10 @@ extern "C" dg_status dg_step_noalloc(const dg_mesh* m, int k, int eq, const dg_f
     StageLauncher L = stage2d_f64_launcher(k, eq, basis);
     if (!L.launch) return DG_ERR_UNSUPPORTED;
     const int nstrips = (m->nx + STRIP_OUT - 1) / STRIP_OUT;
-    int wpb = (int)((200 * 1024 - 256) / L.slot_bytes_per_warp);
-    if (wpb > 8) wpb = 8;
-    if (wpb < 1) return DG_ERR_UNSUPPORTED;
-    wpb = default_block_warps(L, wpb);
+    const TileShape tile = tile_shape(L, nstrips, m->ny, true, 0, 0);
+    if (tile.warps < 1) return DG_ERR_UNSUPPORTED;
+    const int wpb = tile.warps, H = tile.rows;
     const size_t smem = 256 + L.slot_bytes_per_warp * wpb;
-    if (L.set_smem(smem) != cudaSuccess) return DG_ERR_CUDA;
-    int H = default_chunk_rows(L, nstrips, m->ny, wpb, 32u * wpb, smem);
-    if (H > m->ny) H = m->ny;
     const int nchunks = (m->ny + H - 1) / H;
     const long long nw = (long long)nstrips * nchunks;
     for (int s = 0; s < 3; ++s) {

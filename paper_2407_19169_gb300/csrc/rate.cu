@@ -3,10 +3,10 @@
 // points; the first step's dt comes from it (later steps take theirs inside the last stage).
 //
 // The maximum is formed in FP64 whatever the storage, and FP64 arithmetic is 1/63 of FP32's here, so
-// each warp first brackets every rate of its cells in FP32 (an upper and a lower bound that allow for
+// each block first brackets every rate of its cells in FP32 (an upper and a lower bound that allow for
 // the rounding of the coefficients, of the evaluation and of the flux functions) and evaluates in FP64
 // only cells whose upper bound reaches the largest lower bound seen: the result is the FP64 maximum,
-// from a few cells per warp. Cells without higher modes take their average alone. What bounds it then
+// from a few cells per block. Cells without higher modes take their average alone. What bounds it then
 // is two FP32 passes over the points; before, each point cost an FP64 Legendre recurrence with
 // divisions (2D Q2, 1024^2, 21 points: 7.4 ms, more than eight whole steps).
 #include "dg_internal.h"
@@ -64,9 +64,14 @@ static __device__ __forceinline__ RateBounds rate_bounds(const float (&w)[NV], c
   return r;
 }
 
-static __device__ __forceinline__ float warp_max_f(float x) {
+static __device__ __forceinline__ float block_max(float x) {
+  __shared__ float part[8];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = x;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) x = fmaxf(x, part[w]);
   return x;
 }
 
@@ -114,7 +119,7 @@ __global__ void __launch_bounds__(256) rate_averages_kernel(const AuxGeom g, con
       for (int v = 0; v < NV; ++v) ub[v] = rate_avg(g, st, v, c);
       floor_ = fmaxf(floor_, bounds(ub).lo);
     }
-    floor_ = fmaxf(warp_max_f(floor_), rate_so_far(sc, slot));
+    floor_ = fmaxf(block_max(floor_), rate_so_far(sc, slot));
   }
   double r = 0.0;
   bool ok = true;
@@ -187,7 +192,7 @@ __global__ void __launch_bounds__(256) rate_points_kernel(const AuxGeom g, const
   };
   float floor_ = 0.f;
   for (long long c = i0; c < g.ncell; c += step) floor_ = fmaxf(floor_, bounds(c).lo);
-  floor_ = fmaxf(warp_max_f(floor_), rate_so_far(sc, slot));
+  floor_ = fmaxf(block_max(floor_), rate_so_far(sc, slot));
   double r = 0.0;
   bool ok = true;
   for (long long c = i0; c < g.ncell; c += step) {

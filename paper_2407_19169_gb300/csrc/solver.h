@@ -31,6 +31,7 @@ struct dg_solver {
   int nstrips, nchunks, nwarps1d;
   bool whole_step;          // 1D: one launch per step (step1d_kernel) instead of one per stage
   long long ntiles1d;       // its tiles
+  bool own_tile;            // 2D: the rows per chunk are the library's choice
   cudaGraphExec_t pair_exec;
   bool pair_ready;
   long long pair_launches;  // kernel nodes in the step-pair graph

@@ -538,7 +538,10 @@ struct Stage1D {
     for (int i = 0; i < NP_LIM; ++i) {
       T w[NV];
       value(i, w);
-      if (pressure_of<NV>(w, gm1) < eps) th2 = pp_segment<NV>(ub, w, eps, gm1, th2);
+      if (pressure_of<NV>(w, gm1) < eps) {
+        const T t = pp_segment<NV>(ub, w, eps, gm1);
+        th2 = t < th2 ? t : th2;
+      }
     }
     if (th2 < T(1)) {
 #pragma unroll

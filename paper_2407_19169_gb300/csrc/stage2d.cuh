@@ -891,6 +891,7 @@ struct Stage2D {
     T* wq = ws + SLOT_WORDS;                                      // Q[v][l-1] of the next row to filter
     T* weta = wq + NV * LMAX * 32;                                // hybrid: eta of the next row, partial
     T my_eta = T(0);
+    T top_rate = T(0.95) * (T)a.cfl / dt;                         // limiter: see limit_and_rate
     const int nx = a.nx, ny = a.ny;
     // mesh and physics constants from the kernel parameters (stage2d_consts)
     const Consts2D<T>& KC = consts_of(a);
@@ -1412,10 +1413,23 @@ struct Stage2D {
             }
           } else if (a.filter_on) {
             T fac[LMAX + 1];
-            const T damp = -(invH2 * dt);
+            if constexpr (PR::MIXED) {
+              // exp(-sigma dt) as 2^(-sigma dt log2 e) by the hardware's approximate exponential
+              // (about 2 ulp; a damping factor in (0, 1])
+              const T dtl = dt * T(1.4426950408889634);
 #pragma unroll
-            for (int l = 1; l <= LMAX; ++l) sig[l] *= damp;
-            exp_damp(sig, fac);
+              for (int l = 1; l <= LMAX; ++l) {
+                const float x = -(sig[l] * invH2) * dtl;
+                float f;
+                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(x));
+                fac[l] = f;
+              }
+            } else {
+              const T damp = -(invH2 * dt);
+#pragma unroll
+              for (int l = 1; l <= LMAX; ++l) sig[l] *= damp;
+              exp_damp(sig, fac);
+            }
             if (a.filter_on == FILT_GLOBAL) {
               // one coefficient for every mode, from the jumps of all derivative orders (Eq. para:damp)
 #pragma unroll
@@ -1443,7 +1457,8 @@ struct Stage2D {
           }
           T rate_pts = T(0);
           if constexpr (LIM) {
-            if (a.positivity) rate_pts = limit_and_rate(uo, out_lane, ws, sl2, gam, gm1, inv_hx, inv_hy);
+            if (a.positivity) rate_pts = limit_and_rate(uo, out_lane, a.stage == 2, ws, sl2, gam, gm1, inv_hx, inv_hy, (T)a.hx, (T)a.hy,
+                                                       top_rate);
           }
           if (out_lane) {
             ST::store(a.uout, a.ncell, cell2, uo, lo);
@@ -1591,14 +1606,14 @@ struct Stage2D {
   //
   // Bound by instruction issue. Nearly every cell is admissible, so one sum-factorised pass over the
   // points takes the smallest density and pressure and the rate together (a step of a 1024^2 Q2 solve
-  // with the limiter 819 -> 524 us, without it 425; Q3 at 512^2 702 -> 537, without it 486; FP64 Q2 at
+  // with the limiter 819 -> 550 us, without it 425; Q3 at 512^2 702 -> 572, without it 486; FP64 Q2 at
   // 128^2 4137 -> 2970; before: a dense sum per point, once for the density, once for the pressure and
   // once for the rate); the cells of a warp that fail are limited one after the other by
   // the whole warp, a lane per point (limit_cells), so that a strip along a near-vacuum front, whose
   // every row has such cells, does not hold its launch up. Called by all lanes of the warp; ws, slot:
   // a row slot that holds nothing any more (the cells are passed through it).
-  static __device__ __forceinline__ T limit_and_rate(T (&uo)[NV][NM], bool active, T* ws, int slot, T gam, T gm1,
-                                                     T ihx, T ihy) {
+  static __device__ __forceinline__ T limit_and_rate(T (&uo)[NV][NM], bool active, bool want_rate, T* ws, int slot,
+                                                     T gam, T gm1, T ihx, T ihy, T hx, T hy, T& top) {
     if constexpr (EQ != EQ_EULER) {
       return T(0);
     } else {
@@ -1612,7 +1627,8 @@ struct Stage2D {
         pmin = fmin(pmin, p);
         rate = nan_max(euler_rate(w, inv, p, gam, ihx, ihy), rate);
       });
-      const bool fails = active && eps > T(0) && eps_r > T(0) && (rmin < eps_r || pmin < eps);
+      // the margins with some slack: limit_cells decides with sums in a fixed order
+      const bool fails = active && eps > T(0) && eps_r > T(0) && (rmin < T(1.01) * eps_r || pmin < T(1.01) * eps);
       const unsigned mask = __ballot_sync(0xffffffffu, fails);
       if (mask) {
         const int lane = threadIdx.x & 31;
@@ -1624,19 +1640,66 @@ struct Stage2D {
         }
         __syncwarp();
         T th1 = T(1), th2 = T(1);
-        limit_cells(mask, ws, slot, eps_r, eps, gam, gm1, ihx, ihy, th1, th2, rate);
+        limit_cells(mask, ws, slot, eps_r, eps, gam, gm1, hx, hy, th1, th2, rate);
         if (fails) {
-          const T th = th1 * th2;
 #pragma unroll
           for (int m = 1; m < NM; ++m) {
-            uo[0][m] *= th;
+            uo[0][m] *= th1;
 #pragma unroll
-            for (int v = 1; v < NV; ++v) uo[v][m] *= th2;
+            for (int v = 0; v < NV; ++v) uo[v][m] *= th2;
           }
         }
       }
-      return rate;
+      if constexpr (!PR::MIXED) {
+        return rate;
+      } else {
+        // The FP32 form's dt follows the digits of the rate at the point that gives the maximum, and next
+        // to vacuum those digits depend on the order of the sum. So for cells near the maximum the rate is
+        // formed again by the plain sum mode by mode (as limit_cells forms it); top is the warp's largest
+        // rate so far, from a start a little below u^n's rate. Only the last stage's rate is used.
+        if (!want_rate) return T(0);
+        const bool may = active && !fails && !(T(1.0001) * rate < top);
+        const unsigned some = __ballot_sync(0xffffffffu, may);
+        if (some) {
+          T cell[NV][NM];
+#pragma unroll
+          for (int v = 0; v < NV; ++v)
+#pragma unroll
+            for (int m = 0; m < NM; ++m) cell[v][m] = uo[v][m];
+          const T plain = plain_rate(cell, gam, gm1, hx, hy);
+          if (may) rate = plain;
+        }
+        if (some | mask) {
+          T r = active ? rate : T(0);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) r = nan_max(__shfl_xor_sync(0xffffffffu, r, o), r);
+          top = nan_max(r, top);
+        }
+        return rate;
+      }
     }
+  }
+  // The largest CFL rate over the limiter's points of a cell, each point value summed mode by mode.
+  static __device__ __noinline__ T plain_rate(const T (&u)[NV][NM], T gam, T gm1, T hx, T hy) {
+    const carr<T, NP_LIM * NM>& C = lim_table<K, BASIS, T>;
+    T rate = T(0);
+#pragma unroll 2
+    for (int i = 0; i < NP_LIM; ++i) {
+      T w[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) w[v] = u[v][0];
+#pragma unroll
+      for (int m = 1; m < NM; ++m) {
+        const T c = C[i * NM + m];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) w[v] = tfma(c, u[v][m], w[v]);
+      }
+      T bx, by, invH;
+      bool ph;
+      avg_params<EQ, 2>(w, gam, gm1, T(0), T(0), bx, by, invH, ph);
+      rate = nan_max(bx / hx + by / hy, rate);
+    }
+    return rate;
   }
   // Admissibility margins, relative to the cell average in both precisions (as the oracle):
   // rho(x) >= 1e-3 rho_bar and p(x) >= min(1e-3 (rho_bar + |E_bar|), rho_bar, p_bar). Relative
@@ -1658,8 +1721,8 @@ struct Stage2D {
   // theta_1, theta_2 and the limited cell's rate for the cells of the lanes in mask, which hold their
   // coefficients in row slot `slot`: lane i evaluates point i (and i + 32) of each cell and solves for
   // its own largest admissible theta_2. Rolled, so that the rare path costs the others no registers.
-  static __device__ __noinline__ void limit_cells(unsigned mask, T* ws, int slot, T eps_r_, T eps_, T gam,
-                                                  T gm1, T ihx, T ihy, T& th1_, T& th2_, T& rate_) {
+  static __device__ __noinline__ void limit_cells(unsigned mask, T* ws, int slot, T eps_r_, T eps_, T gam, T gm1,
+                                                  T hx, T hy, T& th1_, T& th2_, T& rate_) {
     constexpr int PER = (NP_LIM + 31) / 32;
     const int lane = threadIdx.x & 31;
     const carr<T, NP_LIM * NM>& C = lim_table<K, BASIS, T>;
@@ -1675,44 +1738,50 @@ struct Stage2D {
       const int j = __ffs(mask) - 1;
       mask &= mask - 1;
       const T eps_r = __shfl_sync(0xffffffffu, eps_r_, j), eps = __shfl_sync(0xffffffffu, eps_, j);
-      T ub[NV], w[PER][NV], th1 = T(1), th2 = T(1);
+      T ub[NV], th1 = T(1), th2 = T(1);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        ub[v] = *slot_ptr(ws, slot, v, 0, j);
+      for (int v = 0; v < NV; ++v) ub[v] = *slot_ptr(ws, slot, v, 0, j);
+      // the point values of variables v >= first with the modes scaled by theta_1 (density) and theta_2
+      auto values = [&](T (&w)[PER][NV], int first, int end) {
 #pragma unroll
-        for (int i = 0; i < PER; ++i) w[i][v] = ub[v];
+        for (int v = 0; v < NV; ++v) {
+          if (v < first || v >= end) continue;
 #pragma unroll
-        for (int m = 1; m < NM; ++m) {
-          const T x = *slot_ptr(ws, slot, v, m, j);
+          for (int i = 0; i < PER; ++i) w[i][v] = ub[v];
 #pragma unroll
-          for (int i = 0; i < PER; ++i) w[i][v] += c[i][m] * x;
+          for (int m = 1; m < NM; ++m) {
+            T x = *slot_ptr(ws, slot, v, m, j);
+            if (v == 0) x = tmul(x, th1);
+            x = tmul(x, th2);
+#pragma unroll
+            for (int i = 0; i < PER; ++i) w[i][v] = tfma(c[i][m], x, w[i][v]);
+          }
         }
-      }
-      // density: rho_bar + theta_1 (rho - rho_bar) = eps_r + theta_1 (rho - rho_min), which keeps the digits
-      // of a density far below the average
-      T low = w[0][0];
+      };
+      T w[PER][NV];
+      values(w, 0, NV);
+      T low = ub[0];
 #pragma unroll
-      for (int i = 1; i < PER; ++i) low = fmin(low, w[i][0]);
+      for (int i = 0; i < PER; ++i) low = fmin(low, w[i][0]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) low = fmin(low, __shfl_xor_sync(0xffffffffu, low, o));
-      const bool thin = low < eps_r;
-      if (thin) th1 = (ub[0] - eps_r) / (ub[0] - low);
-#pragma unroll
-      for (int i = 0; i < PER; ++i) {
-        if (thin) w[i][0] = eps_r + th1 * (w[i][0] - low);
-        if (pressure_of<NV>(w[i], gm1) < eps) th2 = pp_segment<NV>(ub, w[i], eps, gm1, th2);
+      if (low < eps_r) {
+        th1 = (ub[0] - eps_r) / (ub[0] - low);
+        values(w, 0, 1);
       }
 #pragma unroll
+      for (int i = 0; i < PER; ++i)
+        if (pressure_of<NV>(w[i], gm1) < eps) th2 = fmin(th2, pp_segment<NV>(ub, w[i], eps, gm1));
+#pragma unroll
       for (int o = 16; o > 0; o >>= 1) th2 = fmin(th2, __shfl_xor_sync(0xffffffffu, th2, o));
+      if (th2 < T(1)) values(w, 0, NV);
       T rate = T(0);
 #pragma unroll
       for (int i = 0; i < PER; ++i) {
-        T x[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) x[v] = ub[v] + th2 * (w[i][v] - ub[v]);
-        const T inv = arcp(x[0]);
-        const T p = gm1 * (x[3] - T(0.5) * (x[1] * x[1] + x[2] * x[2]) * inv);
-        rate = nan_max(euler_rate(x, inv, p, gam, ihx, ihy), rate);
+        T bx, by, invH;
+        bool ph;
+        avg_params<EQ, 2>(w[i], gam, gm1, T(0), T(0), bx, by, invH, ph);
+        rate = nan_max(bx / hx + by / hy, rate);
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) rate = nan_max(__shfl_xor_sync(0xffffffffu, rate, o), rate);
