@@ -241,6 +241,9 @@ TileShape dgk::tile_shape(const StageLauncher& L, int nstrips, int ny, bool fp64
   int most = (int)((200 * 1024 - 256) / L.slot_bytes_per_warp);
   if (most > 8) most = 8;
   if (most < 1) return TileShape{0, 0};
+  // the kernel's shared-memory limit is one for all its launches: always that of the largest block, so
+  // that no solver's choice takes another's away
+  if (L.set_smem(256 + L.slot_bytes_per_warp * most) != cudaSuccess) return TileShape{0, 0};
   const int nsm = device_sms();
   TileShape best{0, 0};
   double cost = -1.0;
@@ -248,7 +251,6 @@ TileShape dgk::tile_shape(const StageLauncher& L, int nstrips, int ny, bool fp64
     if (warps > 0 ? c != 4 : c > most) continue;
     const int wpb = warps > 0 ? (warps < most ? warps : most) : c;
     const size_t smem = 256 + L.slot_bytes_per_warp * wpb;
-    if (L.set_smem(smem) != cudaSuccess) continue;
     const int bps = L.blocks_per_sm ? L.blocks_per_sm(32u * wpb, smem) : 0;
     if (bps < 1) continue;
     for (int w = 1; w <= 64; ++w) {                     // warps per SM
@@ -263,7 +265,6 @@ TileShape dgk::tile_shape(const StageLauncher& L, int nstrips, int ny, bool fp64
       if (rows > 0 || nch == ny) break;
     }
   }
-  if (best.warps > 0 && L.set_smem(256 + L.slot_bytes_per_warp * best.warps) != cudaSuccess) return TileShape{0, 0};
   return best;
 }
 

@@ -30,6 +30,7 @@ struct BatchInst {
   long long ncell;
   long long item0;     // first work item of this instance within its class
   int nx, ny, bcx, bcy, H, nstrips, nchunks, filter_on, positivity;
+  int group, strips;   // 1D: strips of an item (persistent path) and of the instance
   double hx, hy, gamma, ax, ay, cfl;
   // 1D mesh constants from the host (stage1d_consts)
   double inv_h_d;
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(256) batch1d_kernel(const BatchArgs b) {
     a.gamma = I.gamma;
     a.ax = I.ax;
     a.cfl = I.cfl;
-    a.nwarps = I.nstrips;
+    a.nwarps = I.strips;
     a.positivity = I.positivity;
     a.hybrid = 0;
     a.hyb = HybridOut{};
@@ -438,7 +439,7 @@ __global__ void __launch_bounds__(256) persist1d_kernel(const PersistArgs P) {
       a.gamma = I.gamma;
       a.ax = I.ax;
       a.cfl = I.cfl;
-      a.nwarps = I.nstrips;
+      a.nwarps = I.strips;
       a.positivity = I.positivity;
       a.hybrid = 0;
       a.hyb = HybridOut{};
@@ -452,7 +453,8 @@ __global__ void __launch_bounds__(256) persist1d_kernel(const PersistArgs P) {
       }
       T speed = T(0);
       bool ok = true;
-      S::item(a, dt, w - I.item0, speed, ok);
+      const long long s0 = (w - I.item0) * I.group, s1 = s0 + I.group < I.strips ? s0 + I.group : I.strips;
+      for (long long st = s0; st < s1; ++st) S::item(a, dt, st, speed, ok);
       item_end(I, stage, step, (double)speed * I.inv_h_d, ok);
     }
     persist_arrive(P, I, C, phase);
@@ -635,6 +637,8 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       I.H = s->dim == 2 ? s->H : 1;
       I.nstrips = s->dim == 2 ? s->nstrips : s->nwarps1d;
       I.nchunks = s->dim == 2 ? s->nchunks : 1;
+      I.strips = I.nstrips;
+      I.group = 1;
       I.filter_on = s->filter_on;
       I.positivity = s->positivity;
       I.hx = s->geom.hx;
@@ -693,9 +697,9 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       int maxw = (int)((200 * 1024) / BL[c].warp_bytes);
       if (maxw > 8) maxw = 8;
       int best = -1, bw = 1, bb = 1;
+      e = BL[c].set_smem(BL[c].warp_bytes * maxw);   // one limit for all callers' launches of this kernel
       for (int cand : {4, 2, 8, 1}) {
         if (cand > maxw) continue;
-        if (BL[c].set_smem(BL[c].warp_bytes * cand) != cudaSuccess) continue;
         const int bps = BL[c].blocks_per_sm(32u * cand, BL[c].warp_bytes * cand);
         if (bps * cand > best) {
           best = bps * cand;
@@ -707,15 +711,19 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       cls_cap[c] = (long long)nsm * (bb > 0 ? bb : 1);
       BatchInst* I = host.data() + cls_begin[c];
       const char* own = own_tile.data() + cls_begin[c];
+      // the graph path's warps take ranges of equally many items, the persistent path's one at a time
       double cost = -1.0;
       int rows = 8;
-      for (int h : {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64, 96, 128}) {
+      for (int h = 1; h <= 128; h += h < 32 ? 1 : 4) {
         long long items = 0;
         for (int i = 0; i < cls_count[c]; ++i) {
           const int hi = own[i] ? (h < I[i].ny ? h : I[i].ny) : I[i].H;
           items += (long long)I[i].nstrips * ((I[i].ny + hi - 1) / hi);
         }
-        const double t = tile_cost(items, h, bw, best > 0 ? best : 1, nsm, false);
+        const int fit = best > 0 ? best : 1;
+        const long long per = (items + (long long)nsm * fit - 1) / ((long long)nsm * fit);
+        const double t = persistent ? tile_cost(items, h, bw, fit, nsm, false)
+                                    : per * tile_cost((items + per - 1) / per, h, bw, fit, nsm, false);
         if (cost < 0.0 || t < cost) {
           cost = t;
           rows = h;
@@ -727,11 +735,22 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
         I[i].nchunks = (I[i].ny + I[i].H - 1) / I[i].H;
       }
     }
+    if (c < 3 && persistent) {
+      // 1D: an item of one strip would spend more on the queue and the stage counters than on its 28
+      // cells; as many strips per item as leave two items for each resident warp
+      long long strips = 0;
+      for (int i = cls_begin[c]; i < cls_begin[c] + cls_count[c]; ++i) strips += host[i].strips;
+      long long group = strips / (2 * 16LL * nsm);
+      group = group < 1 ? 1 : (group > 64 ? 64 : group);
+      for (int i = cls_begin[c]; i < cls_begin[c] + cls_count[c]; ++i) {
+        host[i].group = (int)group;
+        host[i].nstrips = (int)((host[i].strips + group - 1) / group);
+      }
+    }
     for (int i = cls_begin[c]; i < cls_begin[c] + cls_count[c]; ++i) {
       host[i].item0 = cls_items[c];
       cls_items[c] += (long long)host[i].nstrips * host[i].nchunks;
     }
-    if (cls_count[c] > 0 && BL[c].set_smem) e = BL[c].set_smem(BL[c].warp_bytes * cls_wpb[c]);
   }
   if (e == cudaSuccess) e = cudaMalloc(&dinst, sizeof(BatchInst) * host.size());
   if (e == cudaSuccess)
@@ -806,7 +825,7 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       const int wpb = c < 3 ? 4 : cls_wpb[c];
       const unsigned block = 32u * wpb;
       const size_t smem = PL.warp_bytes * wpb;
-      e = cudaFuncSetAttribute(PL.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (c >= 3) e = cudaFuncSetAttribute(PL.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
       int bps = 0;
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, PL.fn, (int)block, smem);
       if (e != cudaSuccess) break;

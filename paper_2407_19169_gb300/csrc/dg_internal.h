@@ -28,8 +28,8 @@ struct TileShape {
 // blocks of `warps`; in units of one warp's time per row.
 double tile_cost(long long items, int rows, int warps, int resident, int nsm, bool fp64);
 int device_sms();   // SMs of the current device
-// The cheapest tile; rows, warps > 0: the caller's choice of either. {0, 0} if no block fits. Changes the
-// kernel's dynamic shared-memory limit.
+// The cheapest tile; rows, warps > 0: the caller's choice of either. {0, 0} if no block fits. Raises the
+// kernel's dynamic shared-memory limit to that of its largest block.
 TileShape tile_shape(const StageLauncher& L, int nstrips, int ny, bool fp64, int rows, int warps);
 
 // Instantiation tables (one per kernel file). Return {nullptr} if the combination is not compiled.

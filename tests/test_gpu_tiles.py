@@ -31,3 +31,25 @@ def test_tile_shape_does_not_change_the_result(precision, k):
         u, t = run(tile, precision, k)
         assert t == t_ref, tile
         np.testing.assert_array_equal(u, ref, err_msg=str(tile))
+
+
+@pytest.mark.parametrize("k,limiter", [(2, 1), (3, 1), (2, 0)])
+def test_solvers_with_different_default_tiles_side_by_side(k, limiter):
+    # the default block of a small and of a large mesh differ; each solver's first launches come after
+    # the other was created
+    def make(n):
+        s = N.Solver(dim=2, nx=n, ny=n, k=k, eq=N.EQ_EULER, bc=(N.BC_OUTFLOW,) * 4, precision=N.PREC_FP32_MIXED,
+                     positivity=limiter)
+        s.set_initial(N.IC_QUADRANT2D, I.quadrant_params(1))
+        return s
+    sizes = [40, 90, 214, 300, 64]
+    solvers = [make(n) for n in sizes]
+    for s in solvers + solvers[::-1]:
+        s.advance_steps(3)
+        assert s.sync()[0] == 0
+    for s in solvers:
+        s.set_target(1.0)
+    assert N.batch_run(solvers, 2) == 0
+    assert N.batch_run(solvers, 2, persistent=True) == 0
+    for s in solvers:
+        assert s.sync()[2] == 10
