@@ -40,6 +40,7 @@ struct DevScalars {
   unsigned int is_last;           // current step is clipped to land on T_end
   double dt_cfl;                  // cfl / rate of the state after dt_cfl_step steps (0: not known)
   long long dt_cfl_step;
+  unsigned int rate_floor;        // of a written state's rate (rate.cu): bits of a non-negative float
 };
 
 // Hybrid limiter (Algorithm 1) of one solver: the stage kernel stores the unfiltered DG solution
@@ -469,7 +470,7 @@ __device__ __forceinline__ T pressure_of(const T* w, T gm1) {
 // function of the conservative state, so on the segment p - eps changes sign once.
 // FP32: bisection (30 halvings).
 template <int NV>
-__device__ __forceinline__ float pp_segment(const float (&ub)[NV], const float (&w)[NV], float eps, float gm1) {
+__device__ __noinline__ float pp_segment(const float* ub, const float* w, float eps, float gm1) {
   float lo = 0.f, hi = 1.f;
 #pragma unroll 1
   for (int it = 0; it < 30; ++it) {
@@ -487,7 +488,7 @@ __device__ __forceinline__ float pp_segment(const float (&ub)[NV], const float (
 // side: from there t steps back, twice as far each time, to the first point where the pressure holds.
 // Both loops are bounded; t = 0 (the average itself) always holds.
 template <int NV>
-__device__ __forceinline__ double pp_segment(const double (&ub)[NV], const double (&w)[NV], double eps, double gm1) {
+__device__ __noinline__ double pp_segment(const double* ub, const double* w, double eps, double gm1) {
   double d[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) d[v] = w[v] - ub[v];

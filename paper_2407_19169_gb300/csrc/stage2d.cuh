@@ -199,6 +199,50 @@ struct Store {
       }
     }
   }
+  // Rows staged through shared memory by asynchronous copies (paired layouts of whole float4 planes; Q3's
+  // rows would take the shared memory of its row slots, and the persistent batched kernels share an SM
+  // between classes): a warp's buffer holds VECS planes of 32 cells, each lane copies and reads the words
+  // of its own cell.
+  static constexpr bool STAGED = PAIRED && ((NM - 1) & 1) == 0 && NM <= 9 && !COH;
+  static constexpr int VECS = (NV / 2) * (1 + (NM - 1) / 2);
+  static constexpr int STAGE_WORDS = STAGED ? VECS * 32 * 4 : 0;
+  static __device__ __forceinline__ void stage_row(T* buf, int lane, const void* base, long long ncell, long long c) {
+    const F32Layout L{ncell, NV, NM};
+    const unsigned to = (unsigned)__cvta_generic_to_shared(buf) + 16u * lane;
+#pragma unroll
+    for (int pr = 0; pr < NV / 2; ++pr) {
+      const float4* r = (const float4*)((const float*)base + pr * L.region_words()) + c;
+#pragma unroll
+      for (int q = 0; q <= (NM - 1) / 2; ++q)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + (pr * (VECS / (NV / 2)) + q) * 512u),
+                     "l"(r + ncell * q)
+                     : "memory");
+    }
+  }
+  static __device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+  // all but the last N groups of this lane's copies have arrived
+  template <int N>
+  static __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+  static __device__ __forceinline__ void staged(const T* buf, int lane, T (&u)[NV][NM], T (&lo0)[NV]) {
+    const float4* b = (const float4*)buf + lane;
+#pragma unroll
+    for (int pr = 0; pr < NV / 2; ++pr) {
+      const float4* r = b + pr * (VECS / (NV / 2)) * 32;
+      const float4 a = r[0];
+      u[2 * pr][0] = a.x;
+      u[2 * pr + 1][0] = a.y;
+      lo0[2 * pr] = a.z;
+      lo0[2 * pr + 1] = a.w;
+#pragma unroll
+      for (int q = 0; q < (NM - 1) / 2; ++q) {
+        const float4 x = r[32 * (1 + q)];
+        u[2 * pr][1 + 2 * q] = x.x;
+        u[2 * pr + 1][1 + 2 * q] = x.y;
+        u[2 * pr][2 + 2 * q] = x.z;
+        u[2 * pr + 1][2 + 2 * q] = x.w;
+      }
+    }
+  }
   static __device__ __forceinline__ void store(void* base, long long ncell, long long c,
                                                const T (&u)[NV][NM], const T (&lo0)[NV]) {
     if constexpr (!PR::MIXED) {
@@ -303,7 +347,9 @@ struct Stage2D {
   static constexpr int SLOT_WORDS = PACK ? 32 * LS : 3 * NV * NME * 32;
   // per-warp shared memory: the row slots, the partial damping Q[v][l-1] of one row and the partial
   // jump indicator of one row (hybrid limiter)
-  static constexpr size_t warp_bytes() { return sizeof(T) * (SLOT_WORDS + (NV * LMAX + 1) * 32); }
+  // the staged rows of the stage input and of u^n
+  static constexpr int CARRY_WORDS = (NV * LMAX + (LIM ? 1 : 0)) * 32;
+  static constexpr size_t warp_bytes() { return sizeof(T) * (SLOT_WORDS + CARRY_WORDS + 2 * ST::STAGE_WORDS); }
   static constexpr size_t slot_bytes_per_warp() { return warp_bytes(); }
 
   // Zhang and Shu's Gauss-Lobatto mid-lines: their positivity of the averages uses the Gauss nodes
@@ -890,8 +936,11 @@ struct Stage2D {
     const int lane = threadIdx.x & 31;
     T* wq = ws + SLOT_WORDS;                                      // Q[v][l-1] of the next row to filter
     T* weta = wq + NV * LMAX * 32;                                // hybrid: eta of the next row, partial
+    T* wrow = wq + CARRY_WORDS;                                   // staged rows: the stage input's, u^n's
+    T* wrow_n = wrow + ST::STAGE_WORDS;
     T my_eta = T(0);
-    T top_rate = T(0.95) * (T)a.cfl / dt;                         // limiter: see limit_and_rate
+    const T rate_n = (T)a.cfl / dt;                               // limiter: u^n's rate (see limit_and_rate)
+    TopRate top_rate{T(0), chunk * a.H};
     const int nx = a.nx, ny = a.ny;
     // mesh and physics constants from the kernel parameters (stage2d_consts)
     const Consts2D<T>& KC = consts_of(a);
@@ -946,19 +995,30 @@ struct Stage2D {
 
       // row slots of rows t, t-1, t-2, rotated once per row (row r in slot r mod 3)
       int sl0 = slot_of(yb - 2), sl1 = slot_of(yb - 3), sl2 = slot_of(yb - 4);
+      auto row_of = [&](int r) -> int { return pery ? wrap_near(r, ny) : (r < 0 ? 0 : (r >= ny ? ny - 1 : r)); };
+      if constexpr (ST::STAGED) {
+        ST::stage_row(wrow, lane, a.uin, a.ncell, (long long)row_of(yb - 2) * nx + xc);
+        ST::stage_commit();
+      }
 #pragma unroll 1
       for (int t = yb - 2; t <= ye + 1; ++t) {
         const bool grow = !pery && (t < 0 || t >= ny);
-        const int ty = pery ? wrap_near(t, ny) : (t < 0 ? 0 : (t >= ny ? ny - 1 : t));
+        const int ty = row_of(t);
         const long long cell = (long long)ty * nx + xc;
         T u[NV][NM], lo0[NV];
-        ST::load(a.uin, a.ncell, cell, u, lo0);
-        if constexpr (ST::PAIRED) {
-          // the next row of the stage input, and this row of u^n (read after the volume integral)
-          const int tn = t + 1;
-          const int tyn = pery ? (ty + 1 >= ny ? ty + 1 - ny : ty + 1) : (tn < 0 ? 0 : (tn >= ny ? ny - 1 : tn));
-          ST::prefetch(a.uin, a.ncell, (long long)tyn * nx + xc);
-          if (a.stage > 0) ST::prefetch(a.un, a.ncell, cell);
+        if constexpr (ST::STAGED) {
+          // row t was copied during the previous row; u^n's row is wanted after the volume integral
+          ST::template stage_wait<0>();
+          ST::staged(wrow, lane, u, lo0);
+          if (a.stage > 0 && t >= yb - 1 && t <= ye) ST::stage_row(wrow_n, lane, a.un, a.ncell, cell);
+          ST::stage_commit();
+        } else {
+          ST::load(a.uin, a.ncell, cell, u, lo0);
+          if constexpr (ST::PAIRED) {
+            // the next row of the stage input, and this row of u^n (read after the volume integral)
+            ST::prefetch(a.uin, a.ncell, (long long)row_of(t + 1) * nx + xc);
+            if (a.stage > 0) ST::prefetch(a.un, a.ncell, cell);
+          }
         }
         if (grow || gcol) {
 #pragma unroll
@@ -1058,6 +1118,12 @@ struct Stage2D {
           for (int g = 0; g < NQ; ++g)
 #pragma unroll
             for (int v = 0; v < NV; ++v) topPrev[g][v] = top[g][v];
+        }
+
+        // the buffer's row has been used by the traces: the next row into it
+        if constexpr (ST::STAGED) {
+          if (t <= ye) ST::stage_row(wrow, lane, a.uin, a.ncell, (long long)row_of(t + 1) * nx + xc);
+          ST::stage_commit();
         }
 
         // ---- partial u~ of row t: bottom face, vertical faces, volume, RK combination ----
@@ -1164,7 +1230,14 @@ struct Stage2D {
 
           const int s = sl0;
           T un_[NV][NM], unlo[NV];
-          if (a.stage > 0) ST::load(a.un, a.ncell, cell, un_, unlo);
+          if (a.stage > 0) {
+            if constexpr (ST::STAGED) {
+              ST::template stage_wait<1>();
+              ST::staged(wrow_n, lane, un_, unlo);
+            } else {
+              ST::load(a.un, a.ncell, cell, un_, unlo);
+            }
+          }
           // cell average in double-float from the edge integrals, each formed once per edge:
           // u0 + c0 (un0 - u0) + c1 dt/(2h) (Phi_L - Phi_R + Phi_B [- Phi_T at the next row])
           auto df_average = [&](auto v) -> df {          // (instantiated by the FP32 form only)
@@ -1458,7 +1531,7 @@ struct Stage2D {
           T rate_pts = T(0);
           if constexpr (LIM) {
             if (a.positivity) rate_pts = limit_and_rate(uo, out_lane, a.stage == 2, ws, sl2, gam, gm1, inv_hx, inv_hy, (T)a.hx, (T)a.hy,
-                                                       top_rate);
+                                                       ty2, top_rate);
           }
           if (out_lane) {
             ST::store(a.uout, a.ncell, cell2, uo, lo);
@@ -1487,11 +1560,24 @@ struct Stage2D {
         sl1 = sl0;
         sl0 = sfree;
       }
+      if constexpr (ST::STAGED) ST::template stage_wait<0>();
+    }
+    if constexpr (LIM && PR::MIXED && EQ == EQ_EULER && !OE) {
+      if (a.positivity && a.stage == 2) {
+        const int x = strip * STRIP_OUT - 2 + lane;
+        const int xc = a.bcx == BC_PERIODIC ? ((x % nx) + nx) % nx : (x < 0 ? 0 : (x >= nx ? nx - 1 : x));
+        my_rate_t = nan_max(last_rate(a, top_rate, xc, T(0.5) * rate_n, gam, gm1), my_rate_t);
+      }
     }
     if ((LIM && a.hybrid)) hybrid_max(a.hyb, my_eta);
     if constexpr (OE) oedg_reduce<NV>(a.oe, osum, omax, omin);
   }
 
+  // The largest factorised rate of a lane's cells and its row (positivity limiter, FP32 form).
+  struct TopRate {
+    T rest;
+    int row;
+  };
   // ---- point values of a cell (the positivity limiter's points, the OEDG form's volume points) ----
   // P_l at the nodes x of a column: node x_g of the Gauss rule (N < NQ), +1 (N = NQ), 0 (N = NQ + 1).
   template <int N>
@@ -1613,7 +1699,7 @@ struct Stage2D {
   // every row has such cells, does not hold its launch up. Called by all lanes of the warp; ws, slot:
   // a row slot that holds nothing any more (the cells are passed through it).
   static __device__ __forceinline__ T limit_and_rate(T (&uo)[NV][NM], bool active, bool want_rate, T* ws, int slot,
-                                                     T gam, T gm1, T ihx, T ihy, T hx, T hy, T& top) {
+                                                     T gam, T gm1, T ihx, T ihy, T hx, T hy, int row, TopRate& top) {
     if constexpr (EQ != EQ_EULER) {
       return T(0);
     } else {
@@ -1654,30 +1740,26 @@ struct Stage2D {
         return rate;
       } else {
         // The FP32 form's dt follows the digits of the rate at the point that gives the maximum, and next
-        // to vacuum those digits depend on the order of the sum. So for cells near the maximum the rate is
-        // formed again by the plain sum mode by mode (as limit_cells forms it); top is the warp's largest
-        // rate so far, from a start a little below u^n's rate. Only the last stage's rate is used.
+        // to vacuum those digits depend on the order of the sum. So the factorised sums only choose the
+        // cell of each lane with the largest rate, and last_rate forms it again by the plain sum mode by
+        // mode (as limit_cells does for a cell that fails). Only the last stage's rate is used.
         if (!want_rate) return T(0);
-        const bool may = active && !fails && !(T(1.0001) * rate < top);
-        const unsigned some = __ballot_sync(0xffffffffu, may);
-        if (some) {
-          T cell[NV][NM];
-#pragma unroll
-          for (int v = 0; v < NV; ++v)
-#pragma unroll
-            for (int m = 0; m < NM; ++m) cell[v][m] = uo[v][m];
-          const T plain = plain_rate(cell, gam, gm1, hx, hy);
-          if (may) rate = plain;
+        if (active && !fails && rate > top.rest) {
+          top.rest = rate;
+          top.row = row;
         }
-        if (some | mask) {
-          T r = active ? rate : T(0);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) r = nan_max(__shfl_xor_sync(0xffffffffu, r, o), r);
-          top = nan_max(r, top);
-        }
-        return rate;
+        return fails || rate != rate ? rate : T(0);
       }
     }
+  }
+  // The end of an item (FP32 form): the plain rates of the lanes' cells, from the states just stored, if
+  // they are at least `below` (a part of u^n's rate, under which they will not be the maximum).
+  static __device__ __forceinline__ T last_rate(const Stage2DArgs& a, const TopRate& top, int xc, T below, T gam, T gm1) {
+    if (!__any_sync(0xffffffffu, top.rest >= below)) return top.rest;
+    T cell[NV][NM], lo[NV];
+    Store<PR, NV, NM, true>::load(a.uout, a.ncell, (long long)top.row * a.nx + xc, cell, lo);
+    const T plain = plain_rate(cell, gam, gm1, (T)a.hx, (T)a.hy);
+    return top.rest > T(0) ? plain : T(0);
   }
   // The largest CFL rate over the limiter's points of a cell, each point value summed mode by mode.
   static __device__ __noinline__ T plain_rate(const T (&u)[NV][NM], T gam, T gm1, T hx, T hy) {
