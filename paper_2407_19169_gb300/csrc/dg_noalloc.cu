@@ -53,6 +53,7 @@ __global__ void noalloc_reset(DevScalars* sc) {
     sc->is_last = 0u;
     sc->dt_cfl = 0.0;
     sc->dt_cfl_step = 0;
+    sc->rate_floor = 0u;
   }
 }
 

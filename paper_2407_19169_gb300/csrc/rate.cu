@@ -3,10 +3,10 @@
 // points; the first step's dt comes from it (later steps take theirs inside the last stage).
 //
 // The maximum is formed in FP64 whatever the storage, and FP64 arithmetic is 1/63 of FP32's here, so
-// each block first brackets every rate of its cells in FP32 (an upper and a lower bound that allow for
-// the rounding of the coefficients, of the evaluation and of the flux functions) and evaluates in FP64
-// only cells whose upper bound reaches the largest lower bound seen: the result is the FP64 maximum,
-// from a few cells per block. Cells without higher modes take their average alone. What bounds it then
+// every rate is first bracketed in FP32 (an upper and a lower bound that allow for the rounding of the
+// coefficients, of the evaluation and of the flux functions). One kernel takes the largest lower bound of
+// the mesh, a second evaluates in FP64 only cells whose upper bound reaches it: the result is the FP64
+// maximum, from a few cells. Cells without higher modes take their average alone. What bounds it then
 // is two FP32 passes over the points; before, each point cost an FP64 Legendre recurrence with
 // divisions (2D Q2, 1024^2, 21 points: 7.4 ms, more than eight whole steps).
 #include "dg_internal.h"
@@ -22,12 +22,43 @@ static __device__ inline double rate_avg(const AuxGeom& g, const void* st, int v
   return (double)b[L.word(v, 0, c)] + (double)b[L.word(v, g.nm, c)];
 }
 
-// CFL rate of one state in FP64: beta^x / hx (+ beta^y / hy).
+// CFL rate of one state in FP64, beta^x / hx (+ beta^y / hy), with correctly rounded division and root.
 template <int EQ, int DIM>
 static __device__ __forceinline__ double rate_of(const AuxGeom& g, const double* ub, bool& phys) {
   double bx, by, invH;
-  avg_params<EQ, DIM>(ub, g.gamma, g.gamma - 1.0, g.ax, g.ay, bx, by, invH, phys);
+  if constexpr (EQ == EQ_EULER) {
+    const double inv = 1.0 / ub[0], vx = ub[1] * inv;
+    double p, c;
+    if constexpr (DIM == 1) {
+      p = (g.gamma - 1.0) * (ub[2] - 0.5 * ub[1] * vx);
+      c = sqrt(g.gamma * p * inv);
+      by = 0.0;
+      invH = ub[0] * (1.0 / (ub[2] + p));
+    } else {
+      const double vy = ub[2] * inv;
+      p = (g.gamma - 1.0) * (ub[3] - 0.5 * (ub[1] * vx + ub[2] * vy));
+      c = sqrt(g.gamma * p * inv);
+      by = fabs(vy) + c;
+      invH = ub[0] * (1.0 / (ub[3] + p));
+    }
+    bx = fabs(vx) + c;
+    phys = pos_finite(ub[0]) && pos_finite(p) && pos_finite(bx) && (DIM == 1 || pos_finite(by)) && pos_finite(invH);
+  } else {
+    avg_params<EQ, DIM>(ub, g.gamma, g.gamma - 1.0, g.ax, g.ay, bx, by, invH, phys);
+  }
   return bx / g.hx + (DIM == 2 ? by / g.hy : 0.0);
+}
+
+// P_l(x) by the three-term recurrence.
+static __device__ inline double legendre(int l, double x) {
+  double pm = 1.0, p = x;
+  if (l == 0) return 1.0;
+  for (int j = 1; j < l; ++j) {
+    const double pn = ((2.0 * j + 1.0) * x * p - j * pm) / (j + 1.0);
+    pm = p;
+    p = pn;
+  }
+  return p;
 }
 
 // Bounds of the rate of an Euler state w (NV = 3 or 4) whose variables are off by at most d[v]. lo > 0
@@ -64,15 +95,11 @@ static __device__ __forceinline__ RateBounds rate_bounds(const float (&w)[NV], c
   return r;
 }
 
-static __device__ __forceinline__ float block_max(float x) {
-  __shared__ float part[8];
+// The largest lower bound into sc->rate_floor (bits of a non-negative float), one atomic per warp.
+static __device__ __forceinline__ void floor_end(DevScalars* sc, float x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = x;
-  __syncthreads();
-#pragma unroll
-  for (int w = 0; w < 8; ++w) x = fmaxf(x, part[w]);
-  return x;
+  if ((threadIdx.x & 31) == 0) atomicMax(&sc->rate_floor, __float_as_uint(x));
 }
 
 // Block end: the block's maximum (a NaN is kept) and physicality into the solver's scalars.
@@ -90,14 +117,8 @@ static __device__ __forceinline__ void rate_end(DevScalars* sc, int slot, double
   if (bad && (threadIdx.x & 31) == 0) atomicOr(&sc->err, ERRB_NONPHYS);
 }
 
-// The largest rate found so far by any block: a lower bound of the result.
-static __device__ __forceinline__ float rate_so_far(const DevScalars* sc, int slot) {
-  const double r = __longlong_as_double((long long)((volatile const DevScalars*)sc)->rate_bits[slot]);
-  return r < 3e38 ? (float)r * 0.9999999f : 0.f;
-}
-
-// Rate over the cell averages.
-template <int EQ, int DIM>
+// Rate over the cell averages. BOUND: the first kernel, the lower bounds; else the evaluation.
+template <int EQ, int DIM, bool BOUND>
 __global__ void __launch_bounds__(256) rate_averages_kernel(const AuxGeom g, const void* st, DevScalars* sc, int slot) {
   constexpr int NV = NVars<EQ, DIM>::value;
   const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
@@ -112,15 +133,17 @@ __global__ void __launch_bounds__(256) rate_averages_kernel(const AuxGeom g, con
     }
     return rate_bounds<NV>(w, d, gam, gm1, ihx, ihy);
   };
-  if constexpr (EQ == EQ_EULER) {
+  if constexpr (BOUND) {
     for (long long c = i0; c < g.ncell; c += step) {
       double ub[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) ub[v] = rate_avg(g, st, v, c);
       floor_ = fmaxf(floor_, bounds(ub).lo);
     }
-    floor_ = fmaxf(block_max(floor_), rate_so_far(sc, slot));
+    floor_end(sc, floor_);
+    return;
   }
+  if constexpr (EQ == EQ_EULER) floor_ = __uint_as_float(sc->rate_floor);
   double r = 0.0;
   bool ok = true;
   for (long long c = i0; c < g.ncell; c += step) {
@@ -139,7 +162,7 @@ __global__ void __launch_bounds__(256) rate_averages_kernel(const AuxGeom g, con
 }
 
 // Rate over the averages and the positivity limiter's points (Euler).
-template <int DIM, int K, int BASIS, class PR>
+template <int DIM, int K, int BASIS, class PR, bool BOUND>
 __global__ void __launch_bounds__(256) rate_points_kernel(const AuxGeom g, const void* st, DevScalars* sc, int slot) {
   constexpr int NV = NVars<EQ_EULER, DIM>::value;
   constexpr int NM = DIM == 1 ? K + 1 : Modes<K, BASIS>::NM;
@@ -149,6 +172,33 @@ __global__ void __launch_bounds__(256) rate_points_kernel(const AuxGeom g, const
   using TS = typename PR::T;
   const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
   const float gam = (float)g.gamma, gm1 = (float)(g.gamma - 1.0), ihx = (float)(1.0 / g.hx), ihy = (float)(1.0 / g.hy);
+  // values of the modes at the limiter's points
+  constexpr int NP = DIM == 1 ? S1::NP_LIM : limiter_points(K), NQ = K + 1;
+  __shared__ double phi[NP * NM];
+  for (int e = threadIdx.x; e < NP * NM && !BOUND; e += blockDim.x) {
+    const int i = e / NM, m = e % NM;
+    if constexpr (DIM == 1) {
+      const double x = i < NQ ? GaussRule<NQ>::x(i < NQ ? i : 0) : (i == NQ ? -1.0 : (i == NQ + 1 ? 1.0 : 0.0));
+      phi[e] = legendre(m, x);
+    } else {
+      double x, y;
+      if (i < NQ * NQ) {
+        x = GaussRule<NQ>::x(i / NQ);
+        y = GaussRule<NQ>::x(i % NQ);
+      } else if (i < NQ * NQ + 4 * NQ) {
+        const int d = (i - NQ * NQ) & 3;
+        const double at = GaussRule<NQ>::x((i - NQ * NQ) >> 2);
+        x = d == 0 ? -1.0 : (d == 1 ? 1.0 : at);
+        y = d == 2 ? -1.0 : (d == 3 ? 1.0 : at);
+      } else {
+        const int j = i - NQ * NQ - 4 * NQ;
+        const double at = GaussRule<NQ>::x(j >> 1);
+        x = (j & 1) ? at : 0.0;
+        y = (j & 1) ? 0.0 : at;
+      }
+      phi[e] = legendre(g.mp[m], x) * legendre(g.mq[m], y);
+    }
+  }
   // the bounds of all of a cell's rates; the evaluation's error per variable from the sum of the
   // coefficients' magnitudes (|P_l| <= 1)
   auto bounds = [&](long long c) -> RateBounds {
@@ -190,9 +240,14 @@ __global__ void __launch_bounds__(256) rate_points_kernel(const AuxGeom g, const
     }
     return r;
   };
-  float floor_ = 0.f;
-  for (long long c = i0; c < g.ncell; c += step) floor_ = fmaxf(floor_, bounds(c).lo);
-  floor_ = fmaxf(block_max(floor_), rate_so_far(sc, slot));
+  if constexpr (BOUND) {
+    float lower = 0.f;
+    for (long long c = i0; c < g.ncell; c += step) lower = fmaxf(lower, bounds(c).lo);
+    floor_end(sc, lower);
+    return;
+  }
+  __syncthreads();
+  const float floor_ = __uint_as_float(sc->rate_floor);
   double r = 0.0;
   bool ok = true;
   for (long long c = i0; c < g.ncell; c += step) {
@@ -212,7 +267,6 @@ __global__ void __launch_bounds__(256) rate_points_kernel(const AuxGeom g, const
     r = (rc > r || rc != rc) ? rc : r;
     ok = ok && phys;
     if (!varies) continue;                    // every point value is the average
-    constexpr int NP = DIM == 1 ? S1::NP_LIM : limiter_points(K);
 #pragma unroll 1
     for (int i = 0; i < NP; ++i) {
       double w[NV];
@@ -220,10 +274,7 @@ __global__ void __launch_bounds__(256) rate_points_kernel(const AuxGeom g, const
       for (int v = 0; v < NV; ++v) {
         double x = ub[v];
 #pragma unroll
-        for (int m = 1; m < NM; ++m) {
-          const double phi = DIM == 1 ? lim_table1<K, double>[i * NM + m] : lim_table<K, BASIS, double>[i * NM + m];
-          x += phi * (double)u[v][m];
-        }
+        for (int m = 1; m < NM; ++m) x = fma(phi[i * NM + m], (double)u[v][m], x);
         w[v] = x;
       }
       rc = rate_of<EQ_EULER, DIM>(g, w, pphys);
@@ -234,33 +285,49 @@ __global__ void __launch_bounds__(256) rate_points_kernel(const AuxGeom g, const
 }
 
 namespace {
-using RateKernel = void (*)(AuxGeom, const void*, DevScalars*, int);
-
+// the two kernels of a configuration (scalar laws need no bounds)
+struct RateKernels {
+  void (*bound)(AuxGeom, const void*, DevScalars*, int);
+  void (*evaluate)(AuxGeom, const void*, DevScalars*, int);
+};
+template <int DIM, int K, int BASIS, class PR>
+RateKernels points_kernels() {
+  return {&rate_points_kernel<DIM, K, BASIS, PR, true>, &rate_points_kernel<DIM, K, BASIS, PR, false>};
+}
 template <int DIM, int K, int BASIS>
-RateKernel points_kernel(int prec) {
-  return prec == PREC_F64 ? (RateKernel)&rate_points_kernel<DIM, K, BASIS, PrecF64>
-                          : (RateKernel)&rate_points_kernel<DIM, K, BASIS, PrecF32M>;
+RateKernels points_kernels(int prec) {
+  return prec == PREC_F64 ? points_kernels<DIM, K, BASIS, PrecF64>() : points_kernels<DIM, K, BASIS, PrecF32M>();
 }
 template <int K>
-RateKernel points_kernel(const AuxGeom& g) {
-  if (g.dim == 1) return points_kernel<1, K, BASIS_Q>(g.prec);
-  return g.basis == BASIS_Q ? points_kernel<2, K, BASIS_Q>(g.prec) : points_kernel<2, K, BASIS_P>(g.prec);
+RateKernels points_kernels(const AuxGeom& g) {
+  if (g.dim == 1) return points_kernels<1, K, BASIS_Q>(g.prec);
+  return g.basis == BASIS_Q ? points_kernels<2, K, BASIS_Q>(g.prec) : points_kernels<2, K, BASIS_P>(g.prec);
 }
-RateKernel rate_kernel_of(const AuxGeom& g) {
-  if (g.eq == EQ_EULER) {
-    if (!g.pp) return g.dim == 1 ? (RateKernel)&rate_averages_kernel<EQ_EULER, 1> : (RateKernel)&rate_averages_kernel<EQ_EULER, 2>;
-    return g.k == 1 ? points_kernel<1>(g) : (g.k == 2 ? points_kernel<2>(g) : points_kernel<3>(g));
+template <int EQ>
+RateKernels averages_kernels(int dim) {
+  if constexpr (EQ == EQ_EULER) {
+    if (dim == 1) return {&rate_averages_kernel<EQ, 1, true>, &rate_averages_kernel<EQ, 1, false>};
+    return {&rate_averages_kernel<EQ, 2, true>, &rate_averages_kernel<EQ, 2, false>};
+  } else {
+    if (dim == 1) return {nullptr, &rate_averages_kernel<EQ, 1, false>};
+    return {nullptr, &rate_averages_kernel<EQ, 2, false>};
   }
-  if (g.eq == EQ_BURG)
-    return g.dim == 1 ? (RateKernel)&rate_averages_kernel<EQ_BURG, 1> : (RateKernel)&rate_averages_kernel<EQ_BURG, 2>;
-  return g.dim == 1 ? (RateKernel)&rate_averages_kernel<EQ_ADV, 1> : (RateKernel)&rate_averages_kernel<EQ_ADV, 2>;
+}
+RateKernels rate_kernels_of(const AuxGeom& g) {
+  if (g.eq == EQ_EULER) {
+    if (!g.pp) return averages_kernels<EQ_EULER>(g.dim);
+    return g.k == 1 ? points_kernels<1>(g) : (g.k == 2 ? points_kernels<2>(g) : points_kernels<3>(g));
+  }
+  return g.eq == EQ_BURG ? averages_kernels<EQ_BURG>(g.dim) : averages_kernels<EQ_ADV>(g.dim);
 }
 }  // namespace
 
 cudaError_t launch_rate(const AuxGeom& g, const void* state, DevScalars* sc, int slot, cudaStream_t s) {
   unsigned blocks = (unsigned)((g.ncell + 255) / 256);
   if (blocks > 1216) blocks = 1216;
-  rate_kernel_of(g)<<<blocks, 256, 0, s>>>(g, state, sc, slot);
+  const RateKernels k = rate_kernels_of(g);
+  if (k.bound) k.bound<<<blocks, 256, 0, s>>>(g, state, sc, slot);
+  k.evaluate<<<blocks, 256, 0, s>>>(g, state, sc, slot);
   return cudaGetLastError();
 }
 
