@@ -1,11 +1,11 @@
 // dg_batch.cu — batched stepping of many uneven solves (dg_batch_run).
 //
-// Work decomposition: every solver is an instance; the tile items of an instance are its warp
-// strips (1D) or (strip, row-chunk) tiles (2D), exactly the items its own stage kernel would run.
-// Instances of one (dimension, degree) class share one grid-stride work-list kernel per stage: a
-// warp takes the next item of the class, finds its instance by binary search over the instances'
-// first-item offsets, and runs the same item() body as the single-solve kernel with that instance's
-// dt and buffers. 2D classes are split by the positivity limiter, so that every instance runs the
+// Work decomposition: every solver is an instance; the tile items of an instance are the whole-step
+// tiles of a block (1D) or (strip, row-chunk) tiles of a warp (2D), with the bodies of the single-solve
+// kernels (Stage1D::step_tile, Stage2D::item). Instances of one (dimension, degree) class share one
+// work-list kernel per stage (1D: per step): a warp (1D: a block) takes the next item of the class, finds
+// its instance by binary search over the instances' first-item offsets, and runs it with that
+// instance's dt and buffers. 2D classes are split by the positivity limiter, so that every instance runs the
 // instantiation it runs alone (the one without the limiter code when the limiter is off). Large and small instances therefore share the GPU in proportion to their work.
 //
 // Step control per instance, without inter-block waits: a begin kernel computes each instance's
@@ -30,7 +30,7 @@ struct BatchInst {
   long long ncell;
   long long item0;     // first work item of this instance within its class
   int nx, ny, bcx, bcy, H, nstrips, nchunks, filter_on, positivity;
-  int group, strips;   // 1D: strips of an item (persistent path) and of the instance
+  int group, strips;   // 1D: tiles of an item (persistent path) and of the instance
   double hx, hy, gamma, ax, ay, cfl;
   // 1D mesh constants from the host (stage1d_consts)
   double inv_h_d;
@@ -45,7 +45,6 @@ struct BatchArgs {
   int ninst;
   long long nitems;
   int stage;
-  float c0_hi, c0_lo;      // the stage's c0 as a double-float
 };
 
 __device__ __forceinline__ int find_inst(const BatchInst* inst, int n, long long w) {
@@ -142,67 +141,99 @@ __global__ void __launch_bounds__(256) batch2d_kernel(const BatchArgs b) {
   if (cur >= 0) item_end(b.inst[cur], b.stage, cur_step, racc, okacc);
 }
 
+// 1D instances: whole steps (Stage1D::step_tile), by blocks of STEP1D_THREADS cells of which all but
+// STEP_HALO on each side are output. What a block's threads share.
+constexpr int STEP1D_THREADS = 128;
+constexpr int STEP1D_OUT = STEP1D_THREADS - 2 * STEP_HALO;
+template <class S>
+struct Step1DShared {
+  typename S::T link[LINK_BUFFERS][LINK_WARPS][LINK_WORDS];
+  typename S::Coef coef[3];
+  double dt;
+  long long step, item;
+  int run;
+};
+// Read instance I's step control and form the step's coefficients, by the block's first warp: err may be
+// set by other blocks meanwhile, and every thread of the block has to take the same branch.
+template <class S>
+__device__ __forceinline__ void step1d_control(const BatchInst& I, Step1DShared<S>& sh) {
+  if (threadIdx.x < 32) {
+    volatile DevScalars* vs = I.sc;
+    const bool run = (vs->done | vs->err) == 0u;
+    const double dt = vs->dt;
+    S::step_coef((int)threadIdx.x, dt, I.inv_h_d, sh.coef);
+    const int go = __shfl_sync(0xffffffffu, (int)run, 0);
+    if (threadIdx.x == 0) {
+      sh.run = go;
+      sh.dt = dt;
+      sh.step = vs->step;
+    }
+  }
+}
+__device__ __forceinline__ Stage1DArgs step1d_args(const BatchInst& I, long long step) {
+  Stage1DArgs a;
+  const int p = (int)(step & 1);
+  a.uin = a.un = I.buf[p];
+  a.uout = I.buf[1 - p];
+  a.nx = I.nx;
+  a.ncell = I.ncell;
+  a.h = I.hx;
+  a.bc = I.bcx;
+  a.c0 = 0.0;
+  a.c1 = 1.0;
+  a.stage = 0;
+  a.filter_on = I.filter_on;
+  a.gamma = I.gamma;
+  a.ax = I.ax;
+  a.cfl = I.cfl;
+  a.nwarps = I.strips;
+  a.positivity = I.positivity;
+  a.hybrid = 0;
+  a.hyb = HybridOut{};
+  a.sc = I.sc;
+  a.inv_h_d = I.inv_h_d;
+  a.inv_h_f = I.inv_h_f;
+  a.c0_hi = a.c0_lo = 0.f;
+  return a;
+}
+template <class S>
+__device__ __forceinline__ void step1d_tile(const Stage1DArgs& a, Step1DShared<S>& sh, long long tile,
+                                            typename S::T& speed, bool& ok) {
+  BlockLink<typename S::T> link{sh.link, (int)(threadIdx.x >> 5), STEP1D_THREADS / 32};
+  const typename S::Place pl = S::place(a, (int)(tile * STEP1D_OUT) - STEP_HALO, (int)threadIdx.x, STEP1D_THREADS, STEP_HALO);
+  typename S::T un[S::NV][S::NM], unlo[S::NV];
+  S::ST::load(a.un, a.ncell, pl.cell, un, unlo);
+  S::step_tile(a, sh.coef, (typename S::T)sh.dt, pl, link, un, unlo, speed, ok);
+}
+
+// One step of the class's instances, one launch per step; a block takes a contiguous range of tiles.
 template <int K, int EQ, class PR>
-__global__ void __launch_bounds__(256) batch1d_kernel(const BatchArgs b) {
+__global__ void __launch_bounds__(STEP1D_THREADS) batch1d_kernel(const BatchArgs b) {
   using S = Stage1D<K, EQ, PR>;
   using T = typename PR::T;
-  const long long nwt = (long long)gridDim.x * (blockDim.x >> 5);
-  // each warp takes a contiguous range of items, so consecutive items mostly belong to one
-  // instance and its rate / physicality are folded once per run of items, not once per item
-  const long long per = (b.nitems + nwt - 1) / nwt;
-  const long long w0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
-  const long long w1 = w0 + per < b.nitems ? w0 + per : b.nitems;
+  __shared__ Step1DShared<S> sh;
+  const long long per = (b.nitems + gridDim.x - 1) / gridDim.x;
+  const long long w0 = (long long)blockIdx.x * per, w1 = w0 + per < b.nitems ? w0 + per : b.nitems;
   int cur = -1;
-  long long cur_step = 0;
-  double racc = 0.0;
-  bool okacc = true;
+  T speed = T(0);
+  bool ok = true;
   for (long long w = w0; w < w1; ++w) {
     const int ii = find_inst(b.inst, b.ninst, w);
     if (ii != cur) {
-      if (cur >= 0) item_end(b.inst[cur], b.stage, cur_step, racc, okacc);
+      __syncthreads();                                     // the last tile is done with the coefficients
+      if (cur >= 0 && sh.run) item_end(b.inst[cur], 2, sh.step, (double)speed * b.inst[cur].inv_h_d, ok);
+      __syncthreads();
       cur = ii;
-      cur_step = ((volatile DevScalars*)b.inst[ii].sc)->step;
-      racc = 0.0;
-      okacc = true;
+      step1d_control(b.inst[ii], sh);
+      speed = T(0);
+      ok = true;
+      __syncthreads();
     }
-    const BatchInst& I = b.inst[ii];
-    volatile DevScalars* vs = I.sc;
-    if (vs->done | vs->err) continue;
-    const long long step = vs->step;
-    const double dt = vs->dt;
-    const int p = (int)(step & 1);
-    Stage1DArgs a;
-    a.uin = b.stage == 0 ? I.buf[p] : (b.stage == 1 ? I.buf[1 - p] : I.buf[2]);
-    a.un = I.buf[p];
-    a.uout = b.stage == 1 ? I.buf[2] : I.buf[1 - p];
-    a.nx = I.nx;
-    a.ncell = I.ncell;
-    a.h = I.hx;
-    a.bc = I.bcx;
-    a.c0 = b.stage == 0 ? 0.0 : (b.stage == 1 ? 0.75 : 1.0 / 3.0);
-    a.c1 = b.stage == 0 ? 1.0 : (b.stage == 1 ? 0.25 : 2.0 / 3.0);
-    a.stage = b.stage;
-    a.filter_on = I.filter_on;
-    a.gamma = I.gamma;
-    a.ax = I.ax;
-    a.cfl = I.cfl;
-    a.nwarps = I.strips;
-    a.positivity = I.positivity;
-    a.hybrid = 0;
-    a.hyb = HybridOut{};
-    a.sc = I.sc;
-    a.inv_h_d = I.inv_h_d;
-    a.inv_h_f = I.inv_h_f;
-    a.c0_hi = b.c0_hi;
-    a.c0_lo = b.c0_lo;
-    T speed = T(0);
-    bool ok = true;
-    S::item(a, dt, w - I.item0, speed, ok);
-    const double r = (double)speed * I.inv_h_d;
-    racc = (r > racc || r != r) ? r : racc;
-    okacc = okacc && ok;
+    if (!sh.run) continue;
+    const Stage1DArgs a = step1d_args(b.inst[ii], sh.step);
+    step1d_tile(a, sh, w - b.inst[ii].item0, speed, ok);
   }
-  if (cur >= 0) item_end(b.inst[cur], b.stage, cur_step, racc, okacc);
+  if (cur >= 0 && sh.run) item_end(b.inst[cur], 2, sh.step, (double)speed * b.inst[cur].inv_h_d, ok);
 }
 
 #ifndef DG_BATCH_K
@@ -264,8 +295,9 @@ struct PersistArgs {
   const BatchInst* inst;        // the class's instances, item0 ascending
   PersistCtl* ctl;              // one per instance
   int ninst;
-  long long nitems;             // items of one phase (one stage of every instance)
-  long long total;              // nitems * 3 * steps
+  long long nitems;             // items of one phase of every instance
+  int phases;                   // of a step: 3 stages (2D), 1 (1D)
+  long long total;              // nitems * phases * steps
   long long steps;
   unsigned long long* queue;    // next queue index (zeroed)
   unsigned int* status;         // PERSIST_TIMEOUT when a wait gave up
@@ -331,7 +363,7 @@ __device__ __forceinline__ void persist_arrive(const PersistArgs& P, const Batch
     const unsigned long long items = (unsigned long long)I.nstrips * (unsigned long long)I.nchunks;
     const unsigned long long prev = atomicAdd(&C->arrived, 1ull);
     if (prev + 1 == (unsigned long long)(phase + 1) * items) {
-      if (phase % 3 == 2) persist_step_advance(I, phase / 3 + 1 < P.steps);
+      if (phase % P.phases == P.phases - 1) persist_step_advance(I, phase / P.phases + 1 < P.steps);
       __threadfence();
       atomicExch(&C->released, (unsigned)(phase + 1));
     }
@@ -406,58 +438,42 @@ __global__ void __launch_bounds__(256) persist2d_kernel(const PersistArgs P) {
   }
 }
 
+// 1D: a phase is a whole step, an item a group of tiles, taken by a block.
 template <int K>
-__global__ void __launch_bounds__(256) persist1d_kernel(const PersistArgs P) {
+__global__ void __launch_bounds__(STEP1D_THREADS) persist1d_kernel(const PersistArgs P) {
   using S = Stage1D<K, EQ_EULER, PrecF32M, false, true>;
   using T = float;
+  __shared__ Step1DShared<S> sh;
   for (;;) {
-    const long long k = persist_take(P);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const long long k = persist_take(P);
+      bool go = k < P.total;
+      if (go) {
+        const long long phase = k / P.nitems;
+        const int ii = find_inst(P.inst, P.ninst, k - phase * P.nitems);
+        go = persist_wait(P.ctl + ii, phase, P.status, P.poll_limit);
+        if (go) step1d_control(P.inst[ii], sh);
+      }
+      if (threadIdx.x == 0) sh.item = go ? k : P.total;
+    }
+    __syncthreads();
+    const long long k = sh.item;
     if (k >= P.total) break;
     const long long phase = k / P.nitems, w = k - phase * P.nitems;
     const int ii = find_inst(P.inst, P.ninst, w);
     const BatchInst& I = P.inst[ii];
-    PersistCtl* C = P.ctl + ii;
-    if (!persist_wait(C, phase, P.status, P.poll_limit)) break;
-    const int stage = (int)(phase % 3);
-    volatile DevScalars* vs = I.sc;
-    if (!(vs->done | vs->err)) {
-      const long long step = vs->step;
-      const double dt = vs->dt;
-      const int p = (int)(step & 1);
-      Stage1DArgs a;
-      a.uin = stage == 0 ? I.buf[p] : (stage == 1 ? I.buf[1 - p] : I.buf[2]);
-      a.un = I.buf[p];
-      a.uout = stage == 1 ? I.buf[2] : I.buf[1 - p];
-      a.nx = I.nx;
-      a.ncell = I.ncell;
-      a.h = I.hx;
-      a.bc = I.bcx;
-      a.c0 = stage == 0 ? 0.0 : (stage == 1 ? 0.75 : 1.0 / 3.0);
-      a.c1 = stage == 0 ? 1.0 : (stage == 1 ? 0.25 : 2.0 / 3.0);
-      a.stage = stage;
-      a.filter_on = I.filter_on;
-      a.gamma = I.gamma;
-      a.ax = I.ax;
-      a.cfl = I.cfl;
-      a.nwarps = I.strips;
-      a.positivity = I.positivity;
-      a.hybrid = 0;
-      a.hyb = HybridOut{};
-      a.sc = I.sc;
-      a.inv_h_d = I.inv_h_d;
-      a.inv_h_f = I.inv_h_f;
-      {
-        const double c0 = a.c0;
-        a.c0_hi = (float)c0;
-        a.c0_lo = (float)(c0 - (double)a.c0_hi);
-      }
+    if (sh.run) {
+      const Stage1DArgs a = step1d_args(I, sh.step);
       T speed = T(0);
       bool ok = true;
-      const long long s0 = (w - I.item0) * I.group, s1 = s0 + I.group < I.strips ? s0 + I.group : I.strips;
-      for (long long st = s0; st < s1; ++st) S::item(a, dt, st, speed, ok);
-      item_end(I, stage, step, (double)speed * I.inv_h_d, ok);
+      const long long t0 = (w - I.item0) * I.group, t1 = t0 + I.group < I.strips ? t0 + I.group : I.strips;
+      for (long long t = t0; t < t1; ++t) step1d_tile(a, sh, t, speed, ok);
+      item_end(I, 2, sh.step, (double)speed * I.inv_h_d, ok);
     }
-    persist_arrive(P, I, C, phase);
+    __threadfence();                                       // this thread's stores before the arrival
+    __syncthreads();
+    if (threadIdx.x < 32) persist_arrive(P, I, P.ctl + ii, phase);
   }
 }
 
@@ -635,7 +651,7 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       I.bcx = s->mesh.bc[0];
       I.bcy = s->dim == 2 ? s->mesh.bc[2] : 0;
       I.H = s->dim == 2 ? s->H : 1;
-      I.nstrips = s->dim == 2 ? s->nstrips : s->nwarps1d;
+      I.nstrips = s->dim == 2 ? s->nstrips : (int)((s->mesh.nx + STEP1D_OUT - 1) / STEP1D_OUT);
       I.nchunks = s->dim == 2 ? s->nchunks : 1;
       I.strips = I.nstrips;
       I.group = 1;
@@ -736,11 +752,11 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       }
     }
     if (c < 3 && persistent) {
-      // 1D: an item of one strip would spend more on the queue and the stage counters than on its 28
-      // cells; as many strips per item as leave two items for each resident warp
+      // 1D: as many tiles per item as leave two items for each resident block, so that the queue and the
+      // counters are paid less often
       long long strips = 0;
       for (int i = cls_begin[c]; i < cls_begin[c] + cls_count[c]; ++i) strips += host[i].strips;
-      long long group = strips / (2 * 16LL * nsm);
+      long long group = strips / (2 * 4LL * nsm);
       group = group < 1 ? 1 : (group > 64 ? 64 : group);
       for (int i = cls_begin[c]; i < cls_begin[c] + cls_count[c]; ++i) {
         host[i].group = (int)group;
@@ -771,27 +787,22 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
     for (int stage = 0; stage < 3 && ce == cudaSuccess; ++stage) {
       ce = cudaEventRecord(fork, main);
       for (int c = 0; c < NCLS && ce == cudaSuccess; ++c) {
-        if (cls_count[c] == 0) continue;
+        if (cls_count[c] == 0 || (c < 3 && stage > 0)) continue;      // 1D: the whole step beside the three stages
         BatchArgs b;
         b.inst = dinst + cls_begin[c];
         b.ninst = cls_count[c];
         b.nitems = cls_items[c];
         b.stage = stage;
-        {
-          const double c0 = stage == 0 ? 0.0 : (stage == 1 ? 0.75 : 1.0 / 3.0);
-          b.c0_hi = (float)c0;
-          b.c0_lo = (float)(c0 - (double)b.c0_hi);
-        }
-        const int wpb = cls_wpb[c];
+        const int wpb = c < 3 ? 1 : cls_wpb[c];
+        const unsigned block = c < 3 ? STEP1D_THREADS : 32u * wpb;
         long long blocks = (cls_items[c] + wpb - 1) / wpb;
-        if (blocks > cls_cap[c]) blocks = cls_cap[c];   // warps then take contiguous item ranges
+        if (blocks > cls_cap[c]) blocks = cls_cap[c];   // warps (1D: blocks) then take contiguous item ranges
         ce = cudaStreamWaitEvent(side[c], fork, 0);
-        if (ce == cudaSuccess)
-          ce = BL[c].launch(b, (unsigned)blocks, 32u * wpb, BL[c].warp_bytes * wpb, side[c]);
+        if (ce == cudaSuccess) ce = BL[c].launch(b, (unsigned)blocks, block, BL[c].warp_bytes * wpb, side[c]);
         if (ce == cudaSuccess) ce = cudaEventRecord(join[c], side[c]);
       }
       for (int c = 0; c < NCLS && ce == cudaSuccess; ++c)
-        if (cls_count[c] > 0) ce = cudaStreamWaitEvent(main, join[c], 0);
+        if (cls_count[c] > 0 && (c >= 3 || stage == 2)) ce = cudaStreamWaitEvent(main, join[c], 0);
     }
     if (ce == cudaSuccess) {
       batch_end_kernel<<<nb, 128, 0, main>>>(dinst, (int)host.size());
@@ -822,8 +833,8 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
     for (int c = 0; c < NCLS && e == cudaSuccess; ++c) {
       if (cls_count[c] == 0) continue;
       const PersistLauncher PL = persist_launcher(c < 3 ? 1 : 2, c % 3 + 1, c >= 6);
-      const int wpb = c < 3 ? 4 : cls_wpb[c];
-      const unsigned block = 32u * wpb;
+      const int wpb = c < 3 ? 1 : cls_wpb[c];                       // items at a time per block
+      const unsigned block = c < 3 ? STEP1D_THREADS : 32u * wpb;
       const size_t smem = PL.warp_bytes * wpb;
       if (c >= 3) e = cudaFuncSetAttribute(PL.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
       int bps = 0;
@@ -842,7 +853,8 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       P.ctl = dctl + cls_begin[c];
       P.ninst = cls_count[c];
       P.nitems = cls_items[c];
-      P.total = cls_items[c] * 3 * steps;
+      P.phases = c < 3 ? 1 : 3;
+      P.total = cls_items[c] * P.phases * steps;
       P.steps = steps;
       P.queue = dq + c;
       P.status = dstatus;
@@ -872,10 +884,13 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
   if (dinst) cudaFree(dinst);
   if (pscr) cudaFree(pscr);
   if (status != DG_OK) return status;
-  int present = 0;
-  for (int c = 0; c < NCLS; ++c) present += cls_count[c] > 0;
+  int present = 0, nodes = 2;
+  for (int c = 0; c < NCLS; ++c) {
+    present += cls_count[c] > 0;
+    nodes += cls_count[c] > 0 ? (c < 3 ? 1 : 3) : 0;
+  }
   // the graph's kernel nodes once per step; the persistent path's begin kernel and class launches
-  solvers[0]->launches += persistent ? 1 + present : steps * (2 + 3LL * present);
+  solvers[0]->launches += persistent ? 1 + present : steps * (long long)nodes;
   for (int i = 0; i < n; ++i) {
     dg_solver* s = solvers[i];
     if (solver_pull_control(s) != DG_OK) return DG_ERR_CUDA;

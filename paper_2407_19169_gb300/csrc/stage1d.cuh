@@ -1,5 +1,5 @@
-// stage1d.cuh — 1D SSP-RK3 steps with the jump filter: the whole step in one launch (step1d_kernel),
-// and single stages for the batched kernels and the variants that need the whole mesh between stages.
+// stage1d.cuh — 1D SSP-RK3 steps with the jump filter: whole steps (step1d_kernel, the batched kernels),
+// and single stages for the variants that need the whole mesh between stages.
 //
 // Per cell K_j and stage (Section 2.1):
 //   R^l = (2l+1)/h [ sum_q w_q f(u_h(xi_q)) P_l'(xi_q) - f^_{j+1/2} + (-1)^l f^_{j-1/2} ]   (Eq. scheme:DG)
@@ -579,6 +579,46 @@ struct Stage1D {
     stage_end(a.sc, a.stage, ctl, a.cfl, my_speed, a.inv_h_d, my_ok, red);
   }
 
+  // The coefficients of stage `lane` (lanes 0..2) of a step of size dt.
+  static __device__ __forceinline__ void step_coef(int lane, double dt, double inv_h_d, Coef* coef) {
+    if (lane < 3) {
+      const double c0 = lane == 0 ? so_c0(0) : (lane == 1 ? so_c0(1) : so_c0(2));
+      const double c1 = lane == 0 ? so_c1(0) : (lane == 1 ? so_c1(1) : so_c1(2));
+      const float h0 = lane == 0 ? (float)so_c0(0) : (lane == 1 ? (float)so_c0(1) : (float)so_c0(2));
+      const float l0 = lane == 2 ? (float)(so_c0(2) - (double)(float)so_c0(2)) : 0.f;
+      coef[lane] = coef_of_stage(c1 * dt, inv_h_d, c0, df{h0, l0});
+    }
+  }
+  // The step of one tile from u^n in un, unlo (already read); stores it and folds its output cells in.
+  static __device__ __forceinline__ void step_tile(const Stage1DArgs& a, const Coef* coef, T dt, const Place& pl,
+                                                   BlockLink<T>& link, T (&un)[NV][NM], T (&unlo)[NV], T& my_speed,
+                                                   bool& my_ok) {
+    T u[NV][NM], lo[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      lo[v] = unlo[v];
+#pragma unroll
+      for (int l = 0; l < NM; ++l) {
+        if (l > 0 && pl.ghost) un[v][l] = T(0);
+        u[v][l] = un[v][l];
+      }
+    }
+    T bx, rate = T(0), eta;
+#pragma unroll 1
+    for (int s = 0; s < 3; ++s) {
+      bool phys;
+      cell_stage<false>(a, coef[s], s == 0, dt, pl, link, u, lo, un, unlo, bx, phys, eta);
+      if (pl.own && !phys) my_ok = false;
+      if constexpr (EQ == EQ_EULER) {
+        if (a.positivity) rate = limit_and_rate(u, !pl.ghost, (T)a.gamma, (T)(a.gamma - 1.0));
+      }
+    }
+    if (pl.own) {
+      ST::store(a.uout, a.ncell, pl.cell, u, lo);
+      my_speed = nan_max(nan_max(bx, rate), my_speed);
+    }
+  }
+
   // A whole step. A block owns tiles of blockDim.x cells, of which all but STEP_HALO on each side are
   // its output: the three stages run on the block's registers, each using up two cells of halo. The
   // state is read and written once per step (one launch per stage moved it 8 times and paid three
@@ -594,46 +634,17 @@ struct Stage1D {
     // the first tile's state is on its way while the step control is read
     long long tile = blockIdx.x;
     Place pl = place(a, (int)(tile * out) - STEP_HALO, (int)threadIdx.x, (int)blockDim.x, STEP_HALO);
-    T un[NV][NM], unlo[NV], u[NV][NM], lo[NV];
+    T un[NV][NM], unlo[NV];
     ST::load(a.un, a.ncell, pl.cell, un, unlo);
-    const StageCtl ctl = stage_begin(a.sc, 0, a.cfl, [&](int lane, const StageCtl& c) {
-      if (lane < 3) {
-        const double c0 = lane == 0 ? so_c0(0) : (lane == 1 ? so_c0(1) : so_c0(2));
-        const double c1 = lane == 0 ? so_c1(0) : (lane == 1 ? so_c1(1) : so_c1(2));
-        const float h0 = lane == 0 ? (float)so_c0(0) : (lane == 1 ? (float)so_c0(1) : (float)so_c0(2));
-        const float l0 = lane == 2 ? (float)(so_c0(2) - (double)(float)so_c0(2)) : 0.f;
-        coef[lane] = coef_of_stage(c1 * c.dt, a.inv_h_d, c0, df{h0, l0});
-      }
-    });
+    const StageCtl ctl = stage_begin(a.sc, 0, a.cfl,
+                                     [&](int lane, const StageCtl& c) { step_coef(lane, c.dt, a.inv_h_d, coef); });
     if (!ctl.run) return;
     BlockLink<T> link{link_words, (int)(threadIdx.x >> 5), (int)(blockDim.x >> 5)};
     const T dt = (T)ctl.dt;
     T my_speed = T(0);
     bool my_ok = true;
     for (;;) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        lo[v] = unlo[v];
-#pragma unroll
-        for (int l = 0; l < NM; ++l) {
-          if (l > 0 && pl.ghost) un[v][l] = T(0);
-          u[v][l] = un[v][l];
-        }
-      }
-      T bx, rate = T(0), eta;
-#pragma unroll 1
-      for (int s = 0; s < 3; ++s) {
-        bool phys;
-        cell_stage<false>(a, coef[s], s == 0, dt, pl, link, u, lo, un, unlo, bx, phys, eta);
-        if (pl.own && !phys) my_ok = false;
-        if constexpr (EQ == EQ_EULER) {
-          if (a.positivity) rate = limit_and_rate(u, !pl.ghost, (T)a.gamma, (T)(a.gamma - 1.0));
-        }
-      }
-      if (pl.own) {
-        ST::store(a.uout, a.ncell, pl.cell, u, lo);
-        my_speed = nan_max(nan_max(bx, rate), my_speed);
-      }
+      step_tile(a, coef, dt, pl, link, un, unlo, my_speed, my_ok);
       tile += gridDim.x;
       if (tile >= a.nwarps) break;
       pl = place(a, (int)(tile * out) - STEP_HALO, (int)threadIdx.x, (int)blockDim.x, STEP_HALO);
