@@ -671,7 +671,7 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
         t.ax = s->ax;
         t.ay = s->ay;
         t.filter_on = s->filter_on;
-        stage2d_consts(t);
+        stage2d_consts(t, s->k);
         I.cf = t.cf;
         I.cd = t.cd;
       }

@@ -38,6 +38,7 @@ template <class T>
 struct Consts2D {
   T px[4], py[4], wx[7], wy[7];
   T pxy[16], pxy2[16];   // (2/h_x)^a1 (2/h_y)^a2 at [a1 * 4 + a2], and twice that
+  T pxyk2[16];           // pxy2 times P_k^(k) for each order that is the degree k (folded top derivatives)
   T ihx, ihy, gam, gm1, ax, ay;
 };
 
@@ -66,7 +67,7 @@ struct Stage2DArgs {
 
 template <class T>
 __host__ __device__ inline void consts2d_fill(Consts2D<T>& c, double hx, double hy, double gamma, double ax,
-                                              double ay, bool oedg) {
+                                              double ay, bool oedg, int k) {
   c.ihx = (T)(1.0 / hx);
   c.ihy = (T)(1.0 / hy);
   c.gam = (T)gamma;
@@ -87,6 +88,8 @@ __host__ __device__ inline void consts2d_fill(Consts2D<T>& c, double hx, double 
     for (int a2 = 0; a2 < 4; ++a2) {
       c.pxy[a1 * 4 + a2] = (T)(px[a1] * py[a2]);
       c.pxy2[a1 * 4 + a2] = (T)(2.0 * px[a1] * py[a2]);
+      const double top = dend(1, k, k);
+      c.pxyk2[a1 * 4 + a2] = (T)(2.0 * px[a1] * py[a2] * (a1 == k ? top : 1.0) * (a2 == k ? top : 1.0));
     }
   double hmx = 1.0, hmy = 1.0, fm = 1.0;        // h^m, m!
   for (int m = 0; m < 7; ++m) {
@@ -102,11 +105,11 @@ __host__ __device__ inline void consts2d_fill(Consts2D<T>& c, double hx, double 
     hmy *= hy;
   }
 }
-// Fill a.cf and a.cd from a.hx, a.hy, a.gamma, a.ax, a.ay and the filter kind.
-__host__ __device__ inline void stage2d_consts(Stage2DArgs& a) {
+// Fill a.cf and a.cd from a.hx, a.hy, a.gamma, a.ax, a.ay, the filter kind and the degree.
+__host__ __device__ inline void stage2d_consts(Stage2DArgs& a, int k) {
   const bool oedg = a.filter_on == FILT_OEDG;
-  consts2d_fill(a.cf, a.hx, a.hy, a.gamma, a.ax, a.ay, oedg);
-  consts2d_fill(a.cd, a.hx, a.hy, a.gamma, a.ax, a.ay, oedg);
+  consts2d_fill(a.cf, a.hx, a.hy, a.gamma, a.ax, a.ay, oedg, k);
+  consts2d_fill(a.cd, a.hx, a.hy, a.gamma, a.ax, a.ay, oedg, k);
 }
 
 constexpr int STRIP_OUT = 28;  // output columns per warp
@@ -745,8 +748,7 @@ struct Stage2D {
           gauss_moments<1>(FY[v], gy);
 #pragma unroll
           for (int q = 0; q <= K; ++q) {
-            gx[q] *= sx;
-            gy[q] *= sy;
+            gy[q] *= sy;                                          // (unpacked: sx = 1)
           }
           sfor<NM>([&](auto Mi) {
             constexpr int m = decltype(Mi)::value;
@@ -769,6 +771,11 @@ struct Stage2D {
   // factor f applied with the absolute values). P_l^{(r)}(-1) = (-1)^{l+r} P_l^{(r)}(+1), so each
   // end sum is formed once from its even- and odd-degree parts. Horizontal edges are the same with
   // the roles of (p, xi) and (q, eta) exchanged.
+
+  // Without packing (FP64, where each product costs the pipe 64 cycles): the factor P_k^(k) of a k-th
+  // derivative, its only term, goes into the weights (Consts2D::pxyk2).
+  static constexpr bool FOLD = !PACK;
+  static constexpr double de(int l, int r) { return FOLD && r == K ? (l == K ? 1.0 : 0.0) : TB::DE[l * (K + 1) + r]; }
 
   // Compile-time structure: the end sum over p of order a1 at fixed q has terms of parity par.
   static constexpr bool xe(int a1, int q, int par) {
@@ -802,7 +809,7 @@ struct Stage2D {
     sfor<K + 1>([&](auto P) {
       constexpr int pp = decltype(P)::value;
       constexpr int m = TB::MIX[pp * (K + 1) + Q];
-      constexpr double c = TB::DE[pp * (K + 1) + A1];
+      constexpr double c = de(pp, A1);
       if constexpr (pp >= A1 && m >= 0 && c != 0.0) {
         if constexpr ((pp & 1) != 0) od = vmad(w[m], (S)c, od);
         else ev = vmad(w[m], (S)c, ev);
@@ -828,7 +835,7 @@ struct Stage2D {
     sfor<K + 1>([&](auto Q) {
       constexpr int q = decltype(Q)::value;
       constexpr int m = TB::MIX[PD * (K + 1) + q];
-      constexpr double c = TB::DE[q * (K + 1) + A2];
+      constexpr double c = de(q, A2);
       if constexpr (q >= A2 && m >= 0 && c != 0.0) {
         if constexpr ((q & 1) != 0) od = vmad(w[m], (S)c, od);
         else ev = vmad(w[m], (S)c, ev);
@@ -857,7 +864,7 @@ struct Stage2D {
     VT ev = vtraits<VT>::zero(), od = vtraits<VT>::zero();
     sfor<K + 1>([&](auto Q) {
       constexpr int q = decltype(Q)::value;
-      constexpr double d = TB::DE[q * (K + 1) + R];
+      constexpr double d = de(q, R);
       constexpr bool present = DIR == 0 ? xw(NO, q) : yw(NO, q);
       if constexpr (q >= R && d != 0.0 && present) {
         if constexpr ((q & 1) != 0) od = vmad(c[q], (S)d, od);
@@ -949,6 +956,7 @@ struct Stage2D {
     const T inv_hx = KC.ihx, inv_hy = KC.ihy;
     // u~ = u + c0 (u^n - u) + c1 dt R: the edge and volume integrals enter through c1 dt / h
     const T sx = (T)(c1dt * ihx), sy = (T)(c1dt * ihy), c0 = (T)a.c0;
+    const T ryx = (T)(a.hx * ihy);                                // sy / sx
     // double-float coefficients of the cell-average update (computed once, off the cell loop)
     const df dfx = df_from_double(0.5 * c1dt * ihx);
     const df dfy = df_from_double(0.5 * c1dt * ihy);
@@ -1053,13 +1061,13 @@ struct Stage2D {
             } else {
               T Fh[NQ][NV];
 #pragma unroll
-              for (int g = 0; g < NQ; ++g) llf2d<EQ, 1>(topPrev[g], bot[g], Fh[g], gam, gm1, ax, ay);
+              for (int g = 0; g < NQ; ++g) llf2d_twice<EQ, 1>(topPrev[g], bot[g], Fh[g], gam, gm1, ax, ay);
 #pragma unroll
               for (int v = 0; v < NV; ++v) {
                 T F[NQ];
 #pragma unroll
                 for (int g = 0; g < NQ; ++g) F[g] = Fh[g][v];
-                gauss_moments<0>(F, Mh[v]);
+                gauss_moments<0, T, true>(F, Mh[v]);
               }
             }
             // finalise u~ of row t-1 with its top-face term (P_q(+1) = 1)
@@ -1170,7 +1178,7 @@ struct Stage2D {
                 T nb[NV];
 #pragma unroll
                 for (int v = 0; v < NV; ++v) nb[v] = shfl_down_t(tl[g][v], 1);
-                llf2d<EQ, 0>(tr[g], nb, FR[g], gam, gm1, ax, ay);
+                llf2d_twice<EQ, 0>(tr[g], nb, FR[g], gam, gm1, ax, ay);
 #pragma unroll
                 for (int v = 0; v < NV; ++v) FL[g][v] = shfl_up_t(FR[g][v], 1);
               }
@@ -1182,8 +1190,8 @@ struct Stage2D {
                   FRv[g] = FR[g][v];
                   FLv[g] = FL[g][v];
                 }
-                gauss_moments<0>(FRv, MR[v]);
-                gauss_moments<0>(FLv, ML[v]);
+                gauss_moments<0, T, true>(FRv, MR[v]);
+                gauss_moments<0, T, true>(FLv, ML[v]);
               }
             }
           }
@@ -1212,12 +1220,13 @@ struct Stage2D {
           } else {
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
+              // in units of sx (the RK combination below multiplies by it)
               T mh[K + 1], dq[K + 1], sq[K + 1];
 #pragma unroll
               for (int i = 0; i <= K; ++i) {
-                mh[i] = sy * Mh[v][i];
-                dq[i] = sx * (ML[v][i] - MR[v][i]);
-                sq[i] = -sx * (ML[v][i] + MR[v][i]);
+                mh[i] = ryx * Mh[v][i];
+                dq[i] = ML[v][i] - MR[v][i];
+                sq[i] = -(ML[v][i] + MR[v][i]);
               }
 #pragma unroll
               for (int m = 0; m < NM; ++m) {
@@ -1226,7 +1235,7 @@ struct Stage2D {
               }
             }
           }
-          volume(u, acc, sx, sy, gm1, ax, ay);
+          volume(u, acc, PACK ? sx : T(1), PACK ? sy : ryx, gm1, ax, ay);
 
           const int s = sl0;
           T un_[NV][NM], unlo[NV];
@@ -1266,7 +1275,7 @@ struct Stage2D {
                 // u + c0 (u^n - u) + c1 dt R  (= c0 u^n + c1 (u + dt R) with c0 + c1 = 1 kept exact)
                 T val = u[v][m];
                 if (a.stage > 0) val += c0 * (un_[v][m] - u[v][m]);
-                val += (T)MINV[m] * acc[v][m];
+                val += ((T)MINV[m] * sx) * acc[v][m];
                 *slot_ptr(ws, s, v, m, lane) = val;
               }
             }
@@ -1400,8 +1409,8 @@ struct Stage2D {
             // whose guards fail only in the first iteration: -> 0.482 ms. Those writes go to a row
             // slot that the partial stage value of row yb overwrites before it is read. Unguarding
             // the partial stage value itself as well was slower, 0.497 ms)
-            if (PACK || need_v) vertical_jumps(w1, sv, KC.pxy, KC.pxy2);
-            horizontal_jumps(w1, w2, sh, KC.pxy, KC.pxy2);
+            if (PACK || need_v) vertical_jumps(w1, sv, KC.pxy, FOLD ? KC.pxyk2 : KC.pxy2);
+            horizontal_jumps(w1, w2, sh, KC.pxy, FOLD ? KC.pxyk2 : KC.pxy2);
             VG av = z, shc = z;
 #pragma unroll
             for (int l = 0; l <= LMAX; ++l) {
