@@ -202,23 +202,30 @@ struct Store {
       }
     }
   }
-  // Rows staged through shared memory by asynchronous copies (paired layouts of whole float4 planes; Q3's
-  // rows would take the shared memory of its row slots, and the persistent batched kernels share an SM
-  // between classes): a warp's buffer holds VECS planes of 32 cells, each lane copies and reads the words
-  // of its own cell.
-  static constexpr bool STAGED = PAIRED && ((NM - 1) & 1) == 0 && NM <= 9 && !COH;
-  static constexpr int VECS = (NV / 2) * (1 + (NM - 1) / 2);
-  static constexpr int STAGE_WORDS = STAGED ? VECS * 32 * 4 : 0;
+  // Rows staged through shared memory by asynchronous copies, up to nine modes (the rows of more would
+  // take the shared memory of their row slots, and the persistent batched kernels, COH, share an SM
+  // between classes): a warp's buffer holds VECS float4 planes of 32 cells and, with an even number of
+  // modes, a float2 plane per pair of variables; each lane copies and reads the words of its own cell.
+  static constexpr bool STAGED = PAIRED && NM <= 9 && !COH;
+  static constexpr int PVECS = 1 + (NM - 1) / 2;              // float4 planes of a pair
+  static constexpr bool TAIL = ((NM - 1) & 1) != 0;
+  static constexpr int TAIL_AT = (NV / 2) * PVECS * 32 * 4;   // word of the float2 planes
+  static constexpr int STAGE_WORDS = STAGED ? TAIL_AT + (TAIL ? (NV / 2) * 32 * 2 : 0) : 0;
   static __device__ __forceinline__ void stage_row(T* buf, int lane, const void* base, long long ncell, long long c) {
     const F32Layout L{ncell, NV, NM};
     const unsigned to = (unsigned)__cvta_generic_to_shared(buf) + 16u * lane;
+    const unsigned tail = (unsigned)__cvta_generic_to_shared(buf) + 4u * TAIL_AT + 8u * lane;
 #pragma unroll
     for (int pr = 0; pr < NV / 2; ++pr) {
-      const float4* r = (const float4*)((const float*)base + pr * L.region_words()) + c;
+      const float* region = (const float*)base + pr * L.region_words();
+      const float4* r = (const float4*)region + c;
 #pragma unroll
-      for (int q = 0; q <= (NM - 1) / 2; ++q)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + (pr * (VECS / (NV / 2)) + q) * 512u),
-                     "l"(r + ncell * q)
+      for (int q = 0; q < PVECS; ++q)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + (pr * PVECS + q) * 512u), "l"(r + ncell * q)
+                     : "memory");
+      if constexpr (TAIL)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(tail + pr * 256u),
+                     "l"((const float2*)(region + 4 * ncell * PVECS) + c)
                      : "memory");
     }
   }
@@ -230,7 +237,7 @@ struct Store {
     const float4* b = (const float4*)buf + lane;
 #pragma unroll
     for (int pr = 0; pr < NV / 2; ++pr) {
-      const float4* r = b + pr * (VECS / (NV / 2)) * 32;
+      const float4* r = b + pr * PVECS * 32;
       const float4 a = r[0];
       u[2 * pr][0] = a.x;
       u[2 * pr + 1][0] = a.y;
@@ -243,6 +250,11 @@ struct Store {
         u[2 * pr + 1][1 + 2 * q] = x.y;
         u[2 * pr][2 + 2 * q] = x.z;
         u[2 * pr + 1][2 + 2 * q] = x.w;
+      }
+      if constexpr (TAIL) {
+        const float2 y = ((const float2*)(buf + TAIL_AT))[pr * 32 + lane];
+        u[2 * pr][NM - 1] = y.x;
+        u[2 * pr + 1][NM - 1] = y.y;
       }
     }
   }
