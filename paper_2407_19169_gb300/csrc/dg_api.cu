@@ -747,18 +747,23 @@ extern "C" dg_status dg_advance_to(dg_solver* s, double T, long long max_steps, 
   const long long step0 = s->h_sc->step;
   st = set_target(s, T, max_steps);
   if (st != DG_OK) return st;
+  // Steps are enqueued without waiting, and those past T are no-ops on the device that still cost their
+  // launches: a few steps first, then as many as the last step size says are left (200-cell Burgers to
+  // T = 0.1, 176 steps: 3 waits and 179 steps instead of 5 and 248).
   long long chunk = 8;
   for (;;) {
     if (s->h_sc->done || s->h_sc->err) break;
     long long room = step0 + max_steps - s->h_step;
+    if (s->h_sc->step > step0 && s->h_sc->dt > 0.0) {
+      const double left = (T - s->h_sc->t) / s->h_sc->dt;
+      chunk = left < 4096.0 ? (long long)left + 1 : 4096;
+    }
     long long n = chunk < room ? chunk : room;
     if (n <= 0) break;
-    // steps past T are no-ops on the device; the parity record is refreshed by pull_control
     st = enqueue_steps(s, n);
     if (st != DG_OK) return st;
-    st = pull_control(s);
+    st = pull_control(s);      // also refreshes the parity record
     if (st != DG_OK) return st;
-    if (chunk < 4096) chunk *= 2;
   }
   if (steps_taken) *steps_taken = s->h_sc->step - step0;
   if (s->h_sc->err) return DG_ERR_NONPHYSICAL;
