@@ -229,19 +229,14 @@ __device__ __forceinline__ bool not_finite(double x) { return abs_bits(x) >= 0x7
 __device__ __forceinline__ bool not_finite(float x) { return !isfinite(x); }
 __device__ __forceinline__ bool pos_finite(float x) { return x > 0.f && isfinite(x); }
 
-// Damping factors f[l] = exp(x[l]), l = 1..N-1, of x <= 0 that decreases with l. FP32: 2^(x log2 e) by the
-// hardware's approximate exponential (about 2 ulp; a factor in (0, 1]). FP64: where the solution is
+// Damping factors f[l] = exp(x[l]), l = 1..N-1, of x <= 0 that decreases with l. FP64: where the solution is
 // smooth the arguments are tiny, and if all of the warp's are, the Taylor polynomial of degree 6
 // (|x| < 2^-9: the next term is below 2^-75) or 10 (|x| < 2^-4: below 2^-69) is exact to rounding in 6 or
 // 10 instructions instead of the function's 15 or more. Called by all lanes of the warp.
 template <int N>
 __device__ __forceinline__ void exp_damp(const float (&x)[N], float (&f)[N]) {
 #pragma unroll
-  for (int l = 1; l < N; ++l) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x[l] * 1.4426950408889634f));
-    f[l] = y;
-  }
+  for (int l = 1; l < N; ++l) f[l] = expf(x[l]);
 }
 template <int N>
 __device__ __forceinline__ void exp_damp(const double (&x)[N], double (&f)[N]) {
@@ -394,8 +389,10 @@ __device__ __forceinline__ void llf1d_twice(const T* uL, const T* uR, T* fh, T g
     const T cL = asqrt(tmul(tmul(gamma, pL), iL)), cR = asqrt(tmul(tmul(gamma, pR), iR));
     const T a = nan_max(tadd(fabs(vL), cL), tadd(fabs(vR), cR));
     const T s0 = tadd(uL[1], uR[1]);
-    const T s1 = tfma(uL[1], vL, tfma(uR[1], vR, tadd(pL, pR)));
-    const T s2 = tfma(vL, tadd(uL[2], pL), tmul(vR, tadd(uR[2], pR)));
+    const T s1 = sizeof(T) == 8 ? tfma(uL[1], vL, tfma(uR[1], vR, tadd(pL, pR)))
+                                : tadd(tfma(uL[1], vL, pL), tfma(uR[1], vR, pR));
+    const T s2 = sizeof(T) == 8 ? tfma(vL, tadd(uL[2], pL), tmul(vR, tadd(uR[2], pR)))
+                                : tadd(tmul(vL, tadd(uL[2], pL)), tmul(vR, tadd(uR[2], pR)));
     fh[0] = tfma(-a, tadd(uR[0], -uL[0]), s0);
     fh[1] = tfma(-a, tadd(uR[1], -uL[1]), s1);
     fh[2] = tfma(-a, tadd(uR[2], -uL[2]), s2);

@@ -32,6 +32,7 @@ namespace {
 
 constexpr size_t NOALLOC_STATE_BYTES = (size_t)32 << 20;       // two stage states together
 constexpr size_t NOALLOC_SCRATCH_BYTES = NOALLOC_STATE_BYTES + 256;  // + the scalars
+static_assert(sizeof(DevScalars) <= 256, "the scalars' part of the array");
 constexpr int MAX_DEVICES = 64;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];

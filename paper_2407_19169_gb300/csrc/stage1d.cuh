@@ -272,7 +272,11 @@ struct Stage1D {
       const T dif = FR[v] - FL[v], sum = FR[v] + FL[v];
 #pragma unroll
       for (int l = PR::MIXED ? 1 : 0; l < NM; ++l) {
-        const T r = l == 0 ? tmul(T(-0.5), dif) : tfma(T(-0.5), (l & 1) ? sum : dif, M[v][l]);
+        // FP32: one face at a time, which cancels the volume term without rounding (the sum of the two
+        // twice-fluxes would round at twice its size)
+        T r;
+        if constexpr (PR::MIXED) r = tfma((l & 1) ? T(-0.5) : T(0.5), FL[v], tfma(T(-0.5), FR[v], M[v][l]));
+        else r = l == 0 ? tmul(T(-0.5), dif) : tfma(T(-0.5), (l & 1) ? sum : dif, M[v][l]);
         T val = tfma(tmul(k.base, T(2 * l + 1)), r, u[v][l]);
         if (!first) val = tfma(k.c0, tadd(un[v][l], -u[v][l]), val);
         u[v][l] = val;
