@@ -108,11 +108,10 @@ typedef struct {
  *             double-float with compensated error-free updates)
  *   workspace optional caller-owned device buffer of at least dg_workspace_size bytes, aligned to
  *             256 bytes; NULL = the library allocates
- *   tile_rows rows per warp in the 2D stage kernel, 0 = default (the height that minimises the
- *             waves of resident warps times the rows a warp sweeps)
- *   tile_warps warps per thread block of the 2D stage kernel, 0 = default (the block size with the
- *             most resident warps per SM); both are tile-shape knobs for the autotuner, results do
- *             not depend on them
+ *   tile_rows rows per warp in the 2D stage kernel, 0 = default (the height with the least estimated
+ *             time: rounds of resident warps, rows a warp sweeps, warps that share an SM)
+ *   tile_warps warps per thread block of the 2D stage kernel, 0 = default (chosen with the rows);
+ *             both are tile-shape knobs for the autotuner, results do not depend on them
  *   positivity Euler only: 1 = the positivity-preserving limiter of Zhang and Shu after the filter in
  *             every stage (the paper applies it this way in Section 3.2), 0 = off (default): density
  *             is kept >= 1e-3 rho_bar and pressure >= min(1e-3 (rho_bar + |E_bar|), rho_bar, p_bar)
@@ -203,9 +202,9 @@ DG_API dg_status dg_set_target(dg_solver* s, double T_end, long long max_steps);
 
 /* Batched stepping (many uneven solves at once): advance every solver in solvers[0..n-1] by up to
  * `steps` SSP-RK3 steps. Solvers of the same (dimension, degree) class share one work-list kernel
- * per stage whose warps take tile items from all instances of the class; the classes run as
- * parallel branches of one CUDA graph that holds a whole step and is replayed `steps` times on the
- * first solver's stream. Each solver keeps its own dt (its own CFL max) and stop condition
+ * per stage (1D: per step) whose warps (1D: blocks) take tile items from all instances of the class;
+ * the classes run as parallel branches of one CUDA graph that holds a whole step and is replayed `steps`
+ * times on the first solver's stream. Each solver keeps its own dt (its own CFL max) and stop condition
  * (dg_set_target): a solver that reaches its T_end or step limit idles. Results equal those of the
  * same solver stepped alone. Supported: Euler, FP32 form, 1D or 2D Q^k; all on one device.
  * Synchronises; returns DG_ERR_NONPHYSICAL if any solver failed (check each with dg_sync). */
@@ -213,16 +212,16 @@ DG_API dg_status dg_batch_run(dg_solver* const* solvers, int n, long long steps)
 
 /* Batched stepping as dg_batch_run, with the same arguments, classes and results, in one persistent
  * launch per class instead of a replayed per-step graph: each class's kernel runs all `steps` steps of
- * its solvers. Its warps take tile items from a queue ordered by (step, stage, solver, item); before
- * an item a warp waits until every item of that solver's earlier stages has finished (a per-solver
- * counter on the device), and the last item of a solver's step advances its t and step count and
+ * its solvers. Its warps take tile items from a queue ordered by (step, stage, solver, item) (1D: blocks
+ * take whole-step items, ordered by (step, solver, item)); before an item a warp waits until every item
+ * of that solver's earlier stages has finished (a per-solver counter on the device), and the last item of a solver's step advances its t and step count and
  * sets its next dt. Solvers therefore move through their stages independently: a small solver does
  * not wait for a large one. The launches are cooperative (all blocks resident). Every wait polls a
  * bounded number of times (about a second); if one gives up, all warps leave and the call returns
  * DG_ERR_TIMEOUT with the solvers' states undefined (a wait that is not broken lasts at most one
  * stage of its solver). Allocates a small device scratch block (16 bytes per solver) per call.
- * A class's launch runs until its whole queue (steps x 3 x its items) is taken, even after all its
- * solvers have reached their T_end: their items are then skipped, at about a microsecond of a warp
+ * A class's launch runs until its whole queue (steps x 3 x its items, 1D: steps x its items) is taken,
+ * even after all its solvers have reached their T_end: their items are then skipped, at about a microsecond of a warp
  * each, so pass a step count near the one needed (dg_batch_run idles the same way, per step).
  * steps above 2^30 are rejected with DG_ERR_ARG (the per-solver stage counters are 32-bit).
  * Synchronises; DG_ERR_NONPHYSICAL as dg_batch_run. Not while a stream is captured. */

@@ -4,8 +4,9 @@
 // Buffers: three state buffers B0, B1, B2. A step starting from B[p] (p = step parity) runs
 //   stage 0: B[p] -> B[1-p];  stage 1: (B[1-p], B[p]) -> B2;  stage 2: (B2, B[p]) -> B[1-p]
 // so the new state lands in B[1-p] and the input is only read: a failing step leaves the last good
-// state where it was. Two consecutive steps form a fixed launch sequence (6 kernels) that is
-// captured once into a CUDA graph and replayed; dt, t and the stop condition live on the device.
+// state where it was. In 1D one kernel runs the whole step, B[p] -> B[1-p]. Two consecutive steps form a
+// fixed launch sequence (6 kernels, 1D: 2) that is captured once into a CUDA graph and replayed; dt, t and
+// the stop condition live on the device.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>

@@ -5,11 +5,12 @@
 // kernels (Stage1D::step_tile, Stage2D::item). Instances of one (dimension, degree) class share one
 // work-list kernel per stage (1D: per step): a warp (1D: a block) takes the next item of the class, finds
 // its instance by binary search over the instances' first-item offsets, and runs it with that
-// instance's dt and buffers. 2D classes are split by the positivity limiter, so that every instance runs the
-// instantiation it runs alone (the one without the limiter code when the limiter is off). Large and small instances therefore share the GPU in proportion to their work.
+// instance's dt and buffers. 2D classes are split by the positivity limiter, so that every instance runs
+// the instantiation it runs alone (the one without the limiter code when the limiter is off). Large and
+// small instances therefore share the GPU in proportion to their work.
 //
 // Step control per instance, without inter-block waits: a begin kernel computes each instance's
-// dt from its CFL rate max (clipped to its T_end), the three stage launches follow, and an end
+// dt from its CFL rate max (clipped to its T_end), the three stage launches (1D: one) follow, and an end
 // kernel advances t and the step count. A whole step — begin, the classes' stage kernels as
 // parallel graph branches, end — is captured once into a CUDA graph and replayed.
 #include <cuda_runtime.h>
