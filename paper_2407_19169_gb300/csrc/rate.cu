@@ -62,33 +62,40 @@ static __device__ inline double legendre(int l, double x) {
 }
 
 // Bounds of the rate of an Euler state w (NV = 3 or 4) whose variables are off by at most d[v]. lo > 0
-// and up finite only where the state is physical for any values within the bounds; up = NaN or inf
-// where FP32 cannot tell. The factors 1 -+ 1e-5 cover the rounding of the operations below.
+// and up finite only where the state is physical for any values within the bounds and FP32 can tell: the
+// kinetic energy is formed as m (m / rho), which stays in range where the energy does (m^2 of densities
+// of 1e-30 does not), and every quantity on the way has to be far above the smallest normal number, or
+// the lost digits could pass for pressure. Otherwise lo = 0 and up = inf: the cell is evaluated. The
+// factors 1 -+ 1e-5 cover the rounding of the operations below.
 struct RateBounds {
   float lo, up;
 };
 template <int NV>
 static __device__ __forceinline__ RateBounds rate_bounds(const float (&w)[NV], const float (&d)[NV], float gam,
                                                          float gm1, float ihx, float ihy) {
-  const float ilo = arcp(w[0] + d[0]), iup = arcp(w[0] - d[0]);   // bounds of 1 / rho
-  float vlo = 0.f, vup = 0.f, mlo = 0.f, mup = 0.f;
+  constexpr float TINY = 1e-33f;
+  const float rlo = w[0] - d[0], rup = w[0] + d[0];
+  const float ilo = arcp(rup), iup = arcp(rlo);                   // bounds of 1 / rho
+  float vlo = 0.f, vup = 0.f, klo = 0.f, kup = 0.f;
 #pragma unroll
   for (int v = 1; v < NV - 1; ++v) {
     const float a = fmaxf(fabsf(w[v]) - d[v], 0.f), b = fabsf(w[v]) + d[v], ih = v == 1 ? ihx : ihy;
-    vlo += a * ih;
-    vup += b * ih;
-    mlo += a * a;
-    mup += b * b;
+    vlo += a * ilo * ih;
+    vup += b * iup * ih;
+    klo += a * (a * ilo);
+    kup += b * (b * iup);
   }
-  const float sh = NV == 3 ? ihx : ihx + ihy;
-  const float plo = gm1 * (w[NV - 1] - d[NV - 1] - 0.50001f * mup * iup);
-  const float pup = gm1 * (w[NV - 1] + d[NV - 1] - 0.49999f * mlo * ilo);
-  const float clo = asqrt(fmaxf(gam * plo * ilo, 0.f)), cup = asqrt(fmaxf(gam * pup * iup, 0.f));
+  const float sh = NV == 3 ? ihx : ihx + ihy, g2 = gam * gm1;
+  const float elo = w[NV - 1] - d[NV - 1] - 0.50001f * kup;       // p / (gamma - 1)
+  const float eup = w[NV - 1] + d[NV - 1] - 0.49999f * klo;
+  const float slo = elo * ilo, sup = eup * iup;
+  const float clo = asqrt(fmaxf(g2 * slo, 0.f)), cup = asqrt(fmaxf(g2 * sup, 0.f));
   RateBounds r;
-  r.lo = 0.99999f * (vlo * ilo + clo * sh);
-  r.up = 1.00001f * (vup * iup + cup * sh);
-  // not certain to be physical (or not a number): no bounds
-  if (!(w[0] - d[0] > 0.f && plo > 0.f && r.up < 3e38f)) {
+  r.lo = 0.99999f * (vlo + clo * sh);
+  r.up = 1.00001f * (vup + cup * sh);
+  const bool known = rlo > TINY && rup < 1.f / TINY && elo > TINY && slo > TINY && g2 * slo > TINY &&
+                     rlo * clo > TINY && ihx > TINY && (NV == 3 || ihy > TINY) && r.lo > TINY && r.up < 3e38f;
+  if (!known) {
     r.lo = 0.f;
     r.up = INFINITY;
   }

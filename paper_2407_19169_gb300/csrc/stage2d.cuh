@@ -1700,11 +1700,6 @@ struct Stage2D {
     }
   }
 
-  // CFL rate beta^x / hx + beta^y / hy of a point value with the pressure of the state.
-  static __device__ __forceinline__ T euler_rate(const T (&w)[NV], T inv, T p, T gam, T ihx, T ihy) {
-    return fabs(w[1] * inv) * ihx + fabs(w[2] * inv) * ihy + asqrt(gam * p * inv) * (ihx + ihy);
-  }
-
   // Zhang-Shu positivity-preserving limiter on one cell (after the filter, as in Section 3.2 of the
   // paper): density first (theta_1), then pressure (theta_2), checked at the points where the scheme
   // evaluates the polynomial (each_point). Cell averages are not touched. Returns the largest CFL rate
@@ -1728,11 +1723,13 @@ struct Stage2D {
       limiter_margins(uo, gm1, eps_r, eps);
       T rmin = uo[0][0], pmin = INFINITY, rate = T(0);
       each_point<true>(uo, [&](const T (&w)[NV]) {
-        const T inv = arcp(w[0]);
-        const T p = gm1 * (w[3] - T(0.5) * (w[1] * w[1] + w[2] * w[2]) * inv);
+        // the kinetic energy as m (m / rho): m^2 of small densities (1e-30) leaves FP32's range
+        const T inv = arcp(w[0]), vx = w[1] * inv, vy = w[2] * inv;
+        const T p = gm1 * (w[3] - T(0.5) * (w[1] * vx + w[2] * vy));
         rmin = fmin(rmin, w[0]);
         pmin = fmin(pmin, p);
-        rate = nan_max(euler_rate(w, inv, p, gam, ihx, ihy), rate);
+        // CFL rate beta^x / hx + beta^y / hy at the point
+        rate = nan_max(fabs(vx) * ihx + fabs(vy) * ihy + asqrt(gam * p * inv) * (ihx + ihy), rate);
       });
       // the margins with some slack: limit_cells decides with sums in a fixed order
       const bool fails = active && eps > T(0) && eps_r > T(0) && (rmin < T(1.01) * eps_r || pmin < T(1.01) * eps);

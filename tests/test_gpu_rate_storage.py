@@ -58,3 +58,52 @@ def test_storage_round_trip(dim, nx, ny, k, eq, basis):
     lo = (u[:, 0] - hi).astype(np.float32)
     assert np.array_equal(r[:, 0], hi.astype(np.float64) + lo)
     assert np.array_equal(r[:, 1:], u[:, 1:].astype(np.float32).astype(np.float64))
+
+
+# Densities of 1e-30 (intergalactic gas in CGS units), and of 1e-20 and 1e25 with velocities of 1e-12 and
+# 1e10 (FP64; their energies leave FP32's range): squared momenta leave that range long before the rate does.
+@pytest.mark.parametrize("rho,speed,precision", [(1e-30, 1e6, N.PREC_FP64), (1e-30, 1e6, N.PREC_FP32_MIXED),
+                                                 (1e-30, 1.0, N.PREC_FP64), (1e-30, 1.0, N.PREC_FP32_MIXED),
+                                                 (1e-20, 1e-12, N.PREC_FP64), (1e25, 1e10, N.PREC_FP64)])
+@pytest.mark.parametrize("dim,nx,ny", [(1, 300, 1), (2, 20, 15)])
+@pytest.mark.parametrize("limiter", [0, 1])
+def test_first_dt_of_states_far_from_one(rho, speed, precision, dim, nx, ny, limiter):
+    # a fast cold stream (rate 1.5 speed / h) hides the one hot cell at rest (1.6 speed / h) only where its
+    # kinetic energy is lost from its pressure (1.73 in 1D, 1.9 in 2D)
+    p = O.Problem(dim=dim, nx=nx, ny=ny, k=2, eq=O.EQ_EULER, bc=(O.BC_PERIODIC,) * 4, positivity=limiter)
+    u = np.zeros(p.shape)
+    c, v = np.full(nx * ny, 0.5 * speed), np.full(nx * ny, speed)
+    hot = nx * ny // 3
+    c[hot], v[hot] = 1.6 * speed, 0.0
+    u[0, 0] = rho
+    for d in range(dim):
+        u[1 + d, 0] = rho * v
+    u[-1, 0] = rho * (c * c / (1.4 * 0.4) + 0.5 * dim * v * v)
+    if precision == N.PREC_FP32_MIXED:               # averages as the form holds them
+        hi = u.astype(np.float32)
+        u = hi.astype(np.float64) + (u - hi).astype(np.float32)
+    s = N.Solver(dim=dim, nx=nx, ny=ny, k=2, eq=N.EQ_EULER, bc=(N.BC_PERIODIC,) * 4, positivity=limiter,
+                 precision=precision)
+    s.write_state(u)
+    dt = s.step()
+    assert abs(dt - O.dt(p, u)) <= 1e-13 * dt
+
+
+@pytest.mark.parametrize("rho,speed", [(1.0, 1.0), (1e-30, 1e6)])
+@pytest.mark.parametrize("k", [1, 2, 3])
+def test_later_dt_of_states_far_from_one(rho, speed, k):
+    # the rate over the limiter's points that a step leaves for the next (2D, FP32 form): a narrow mesh, where
+    # a warp's lanes see, in one column, rows that vary smoothly from the stream to the hot gas at rest
+    p = O.Problem(dim=2, nx=3, ny=40, k=k, eq=O.EQ_EULER, bc=(O.BC_PERIODIC,) * 4, positivity=1)
+    u = np.zeros(p.shape)
+    part = np.repeat(0.5 + 0.5 * np.cos(2 * np.pi * np.arange(40) / 40), 3)
+    c, v = speed * (1.6 - 1.1 * part), speed * part
+    u[0, 0], u[1, 0], u[2, 0] = rho, rho * v, rho * v
+    u[3, 0] = rho * (c * c / (1.4 * 0.4) + v * v)
+    s = N.Solver(dim=2, nx=3, ny=40, k=k, eq=N.EQ_EULER, bc=(N.BC_PERIODIC,) * 4, positivity=1,
+                 precision=N.PREC_FP32_MIXED, tile_rows=40)
+    s.write_state(u)
+    s.step()
+    after, _ = s.read_state()
+    # FP32 rates of the state as stored
+    assert s.step() == pytest.approx(O.dt(p, after), rel=1e-5)
