@@ -32,6 +32,7 @@ struct BatchInst {
   long long item0;     // first work item of this instance within its class
   int nx, ny, bcx, bcy, H, nstrips, nchunks, filter_on, positivity;
   int group, strips;   // 1D: tiles of an item (persistent path) and of the instance
+  int limited;         // 2D with the positivity limiter: the degree, else 0
   double hx, hy, gamma, ax, ay, cfl;
   // 1D mesh constants from the host (stage1d_consts)
   double inv_h_d;
@@ -57,14 +58,27 @@ __device__ __forceinline__ int find_inst(const BatchInst* inst, int n, long long
   return lo;
 }
 
-// Fold one item's rate max and physicality into its instance (lane 0 of the warp).
-__device__ __forceinline__ void item_end(const BatchInst& I, int stage, long long step, double r, bool ok) {
+// Fold one item's rate max, physicality and (2D limiter) cell of the largest rate into its instance.
+__device__ __forceinline__ void item_end(const BatchInst& I, int stage, long long step, double r, bool ok,
+                                         unsigned long long top = 0ull) {
   r = warp_max(r);
   const unsigned bad = __ballot_sync(0xffffffffu, !ok);
   if ((threadIdx.x & 31) == 0) {
     if (bad) atomicOr(&I.sc->err, ERRB_NONPHYS);
     if (stage == 2) atomic_max_nonneg(&I.sc->rate_bits[(step + 1) & 1], r);
   }
+  if (stage == 2) fold_key(&I.sc->top_cell, top);
+  __syncwarp();
+}
+
+// The end of a step of a limited 2D instance of degree K: one more rate into the new state's, as the last
+// block of a solve alone does (Stage2D::take_top_rate). Called by a warp.
+template <int K>
+__device__ __forceinline__ void fold_top_rate(const BatchInst& I) {
+  const long long st = ((volatile DevScalars*)I.sc)->step + 1;
+  const float r = Stage2D<K, EQ_EULER, BASIS_Q, PrecF32M>::take_top_rate(I.sc, I.buf[st & 1], I.ncell, I.cf.gam,
+                                                                         I.cf.gm1, (float)I.hx, (float)I.hy);
+  if ((threadIdx.x & 31) == 0) atomic_max_nonneg(&I.sc->rate_bits[st & 1], (double)r);
   __syncwarp();
 }
 
@@ -87,14 +101,16 @@ __global__ void __launch_bounds__(256) batch2d_kernel(const BatchArgs b) {
   long long cur_step = 0;
   double racc = 0.0;
   bool okacc = true;
+  unsigned long long top = 0ull;
   for (long long w = w0; w < w1; ++w) {
     const int ii = find_inst(b.inst, b.ninst, w);
     if (ii != cur) {
-      if (cur >= 0) item_end(b.inst[cur], b.stage, cur_step, racc, okacc);
+      if (cur >= 0) item_end(b.inst[cur], b.stage, cur_step, racc, okacc, top);
       cur = ii;
       cur_step = ((volatile DevScalars*)b.inst[ii].sc)->step;
       racc = 0.0;
       okacc = true;
+      top = 0ull;
     }
     const BatchInst& I = b.inst[ii];
     volatile DevScalars* vs = I.sc;
@@ -134,12 +150,12 @@ __global__ void __launch_bounds__(256) batch2d_kernel(const BatchArgs b) {
     double r = 0.0;
     T rt = T(0);
     bool ok = true;
-    S::item(a, dt, (int)(local % I.nstrips), (int)(local / I.nstrips), ws, r, rt, ok);
+    S::item(a, dt, (int)(local % I.nstrips), (int)(local / I.nstrips), ws, r, rt, ok, top);
     if constexpr (PR::MIXED) r = (double)rt;
     racc = (r > racc || r != r) ? r : racc;
     okacc = okacc && ok;
   }
-  if (cur >= 0) item_end(b.inst[cur], b.stage, cur_step, racc, okacc);
+  if (cur >= 0) item_end(b.inst[cur], b.stage, cur_step, racc, okacc, top);
 }
 
 // 1D instances: whole steps (Stage1D::step_tile), by blocks of STEP1D_THREADS cells of which all but
@@ -256,12 +272,19 @@ __global__ void batch_begin_kernel(const BatchInst* inst, int n) {
   sc->is_last = last ? 1u : 0u;
 }
 
-// Per-instance step advance at the end of a step (the single-solve last-block rule).
+// Per-instance step advance at the end of a step (the single-solve last-block rule), a warp per instance.
 __global__ void batch_end_kernel(const BatchInst* inst, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (i >= n) return;
-  DevScalars* sc = inst[i].sc;
+  const BatchInst& I = inst[i];
+  DevScalars* sc = I.sc;
   if (sc->done | sc->err) return;
+  switch (I.limited) {
+    case 1: fold_top_rate<1>(I); break;
+    case 2: fold_top_rate<2>(I); break;
+    case 3: fold_top_rate<3>(I); break;
+  }
+  if ((threadIdx.x & 31) != 0) return;
   const double tn = sc->is_last ? sc->T_end : sc->t + sc->dt;
   const long long st = sc->step + 1;
   sc->t = tn;
@@ -354,20 +377,31 @@ __device__ __forceinline__ void persist_step_advance(const BatchInst& I, bool ne
   sc->is_last = last ? 1u : 0u;
 }
 
-// Arrival of one finished (or skipped) item; the last item of an instance's stage releases it.
+// Arrival of one finished (or skipped) item; the last item of an instance's stage releases it. K > 0: the
+// instances are limited and of degree K.
+template <int K>
 __device__ __forceinline__ void persist_arrive(const PersistArgs& P, const BatchInst& I, PersistCtl* C,
                                                long long phase) {
   __threadfence();   // this lane's stores before the arrival
   __syncwarp();
+  bool complete = false;
   if ((threadIdx.x & 31) == 0) {
     __threadfence();
     const unsigned long long items = (unsigned long long)I.nstrips * (unsigned long long)I.nchunks;
     const unsigned long long prev = atomicAdd(&C->arrived, 1ull);
-    if (prev + 1 == (unsigned long long)(phase + 1) * items) {
-      if (phase % P.phases == P.phases - 1) persist_step_advance(I, phase / P.phases + 1 < P.steps);
-      __threadfence();
-      atomicExch(&C->released, (unsigned)(phase + 1));
+    complete = prev + 1 == (unsigned long long)(phase + 1) * items;
+  }
+  const bool step_end = phase % P.phases == P.phases - 1;
+  if constexpr (K > 0) {
+    if (step_end && __shfl_sync(0xffffffffu, (int)complete, 0)) {
+      __threadfence();   // the other items' stores before the loads of the state
+      fold_top_rate<K>(I);
     }
+  }
+  if (complete) {
+    if (step_end) persist_step_advance(I, phase / P.phases + 1 < P.steps);
+    __threadfence();
+    atomicExch(&C->released, (unsigned)(phase + 1));
   }
   __syncwarp();
 }
@@ -432,10 +466,11 @@ __global__ void __launch_bounds__(256) persist2d_kernel(const PersistArgs P) {
       double r = 0.0;
       T rt = T(0);
       bool ok = true;
-      S::item(a, dt, (int)(local % I.nstrips), (int)(local / I.nstrips), ws, r, rt, ok);
-      item_end(I, stage, step, (double)rt, ok);
+      unsigned long long top = 0ull;
+      S::item(a, dt, (int)(local % I.nstrips), (int)(local / I.nstrips), ws, r, rt, ok, top);
+      item_end(I, stage, step, (double)rt, ok, top);
     }
-    persist_arrive(P, I, C, phase);
+    persist_arrive<LIM ? K : 0>(P, I, C, phase);
   }
 }
 
@@ -474,7 +509,7 @@ __global__ void __launch_bounds__(STEP1D_THREADS) persist1d_kernel(const Persist
     }
     __threadfence();                                       // this thread's stores before the arrival
     __syncthreads();
-    if (threadIdx.x < 32) persist_arrive(P, I, P.ctl + ii, phase);
+    if (threadIdx.x < 32) persist_arrive<0>(P, I, P.ctl + ii, phase);
   }
 }
 
@@ -655,6 +690,7 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       I.nstrips = s->dim == 2 ? s->nstrips : (int)((s->mesh.nx + STEP1D_OUT - 1) / STEP1D_OUT);
       I.nchunks = s->dim == 2 ? s->nchunks : 1;
       I.strips = I.nstrips;
+      I.limited = s->dim == 2 && s->positivity ? s->k : 0;
       I.group = 1;
       I.filter_on = s->filter_on;
       I.positivity = s->positivity;
@@ -806,7 +842,7 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
         if (cls_count[c] > 0 && (c >= 3 || stage == 2)) ce = cudaStreamWaitEvent(main, join[c], 0);
     }
     if (ce == cudaSuccess) {
-      batch_end_kernel<<<nb, 128, 0, main>>>(dinst, (int)host.size());
+      batch_end_kernel<<<(unsigned)((host.size() + 3) / 4), 128, 0, main>>>(dinst, (int)host.size());
       ce = cudaGetLastError();
     }
     e = cudaStreamEndCapture(main, &graph);

@@ -41,6 +41,7 @@ struct DevScalars {
   double dt_cfl;                  // cfl / rate of the state after dt_cfl_step steps (0: not known)
   long long dt_cfl_step;
   unsigned int rate_floor;        // of a written state's rate (rate.cu): bits of a non-negative float
+  unsigned long long top_cell;    // 2D limiter, FP32 form: cell_key of the largest rate so far in the last stage
 };
 
 // Hybrid limiter (Algorithm 1) of one solver: the stage kernel stores the unfiltered DG solution

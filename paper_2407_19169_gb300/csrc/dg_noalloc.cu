@@ -55,6 +55,7 @@ __global__ void noalloc_reset(DevScalars* sc) {
     sc->dt_cfl = 0.0;
     sc->dt_cfl_step = 0;
     sc->rate_floor = 0u;
+    sc->top_cell = 0ull;
   }
 }
 

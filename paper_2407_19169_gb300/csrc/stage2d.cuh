@@ -319,8 +319,9 @@ constexpr carr<T, limiter_points(K) * Modes<K, BASIS>::NM> limiter_values() {
   }
   return t;
 }
+// (In global memory: a warp reads them a lane per point, and the constant cache serves one address at a time.)
 template <int K, int BASIS, class T>
-__constant__ carr<T, limiter_points(K) * Modes<K, BASIS>::NM> lim_table = limiter_values<K, BASIS, T>();
+__device__ const carr<T, limiter_points(K) * Modes<K, BASIS>::NM> lim_table = limiter_values<K, BASIS, T>();
 
 // OE = true: the OEDG form of the damping (DG_FILTER_OEDG): the kernel stores u~ unfiltered with the
 // jump sums A_v(l) and the reductions of OedgOut, and the OEDG filter kernel applies the damping.
@@ -944,9 +945,10 @@ struct Stage2D {
 
   // One tile item: strip `strip` (28 output columns) and row chunk `chunk` of one instance, with step
   // size dtd. ws: this warp's row slots and Q area in shared memory. The output cells' max CFL rate
-  // and physicality are folded into my_rate (FP64 form) / my_rate_t (FP32 form) and my_ok.
+  // and physicality are folded into my_rate (FP64 form) / my_rate_t (FP32 form) and my_ok; TOP: the cell
+  // with the lane's largest rate over the limiter's points into my_top (see limit_and_rate).
   static __device__ void item(const Stage2DArgs& a, double dtd, int strip, int chunk, T* ws,
-                              double& my_rate, T& my_rate_t, bool& my_ok) {
+                              double& my_rate, T& my_rate_t, bool& my_ok, unsigned long long& my_top) {
     constexpr carr<int, NM> PP = TB::PP;
     constexpr carr<int, NM> QQ = TB::QQ;
     constexpr carr<double, NM> MINV = TB::MINV;
@@ -958,8 +960,7 @@ struct Stage2D {
     T* wrow = wq + CARRY_WORDS;                                   // staged rows: the stage input's, u^n's
     T* wrow_n = wrow + ST::STAGE_WORDS;
     T my_eta = T(0);
-    const T rate_n = (T)a.cfl / dt;                               // limiter: u^n's rate (see limit_and_rate)
-    TopRate top_rate{T(0), chunk * a.H};
+    TopRow top_row{T(0), 0};
     const int nx = a.nx, ny = a.ny;
     // mesh and physics constants from the kernel parameters (stage2d_consts)
     const Consts2D<T>& KC = consts_of(a);
@@ -1552,7 +1553,7 @@ struct Stage2D {
           T rate_pts = T(0);
           if constexpr (LIM) {
             if (a.positivity) rate_pts = limit_and_rate(uo, out_lane, a.stage == 2, ws, sl2, gam, gm1, inv_hx, inv_hy, (T)a.hx, (T)a.hy,
-                                                       ty2, top_rate);
+                                                       ty2, top_row);
           }
           if (out_lane) {
             ST::store(a.uout, a.ncell, cell2, uo, lo);
@@ -1583,20 +1584,23 @@ struct Stage2D {
       }
       if constexpr (ST::STAGED) ST::template stage_wait<0>();
     }
-    if constexpr (LIM && PR::MIXED && EQ == EQ_EULER && !OE) {
-      if (a.positivity && a.stage == 2) {
-        const int x = strip * STRIP_OUT - 2 + lane;
-        const int xc = a.bcx == BC_PERIODIC ? ((x % nx) + nx) % nx : (x < 0 ? 0 : (x >= nx ? nx - 1 : x));
-        my_rate_t = nan_max(last_rate(a, top_rate, xc, T(0.5) * rate_n, gam, gm1), my_rate_t);
+    if constexpr (TOP) {
+      if (top_row.rate > T(0)) {
+        // (a lane with a rate has its own column: x = strip * STRIP_OUT - 2 + lane)
+        const long long cell = (long long)top_row.row * nx + (strip * STRIP_OUT - 2 + lane);
+        const unsigned long long key = cell_key(top_row.rate, cell);
+        my_top = key > my_top ? key : my_top;
       }
     }
     if ((LIM && a.hybrid)) hybrid_max(a.hyb, my_eta);
     if constexpr (OE) oedg_reduce<NV>(a.oe, osum, omax, omin);
   }
 
-  // The largest factorised rate of a lane's cells and its row (positivity limiter, FP32 form).
-  struct TopRate {
-    T rest;
+  // The limiter in the FP32 form: its last stage leaves the cell with the largest rate (limit_and_rate).
+  static constexpr bool TOP = LIM && PR::MIXED && EQ == EQ_EULER && !OE;
+  // The largest factorised rate of a lane's cells and its row.
+  struct TopRow {
+    T rate;
     int row;
   };
   // ---- point values of a cell (the positivity limiter's points, the OEDG form's volume points) ----
@@ -1715,7 +1719,7 @@ struct Stage2D {
   // every row has such cells, does not hold its launch up. Called by all lanes of the warp; ws, slot:
   // a row slot that holds nothing any more (the cells are passed through it).
   static __device__ __forceinline__ T limit_and_rate(T (&uo)[NV][NM], bool active, bool want_rate, T* ws, int slot,
-                                                     T gam, T gm1, T ihx, T ihy, T hx, T hy, int row, TopRate& top) {
+                                                     T gam, T gm1, T ihx, T ihy, T hx, T hy, int row, TopRow& top) {
     if constexpr (EQ != EQ_EULER) {
       return T(0);
     } else {
@@ -1723,13 +1727,15 @@ struct Stage2D {
       limiter_margins(uo, gm1, eps_r, eps);
       T rmin = uo[0][0], pmin = INFINITY, rate = T(0);
       each_point<true>(uo, [&](const T (&w)[NV]) {
-        // the kinetic energy as m (m / rho): m^2 of small densities (1e-30) leaves FP32's range
-        const T inv = arcp(w[0]), vx = w[1] * inv, vy = w[2] * inv;
-        const T p = gm1 * (w[3] - T(0.5) * (w[1] * vx + w[2] * vy));
+        // the kinetic energy as m (m / rho): m^2 of small densities (1e-30) leaves FP32's range. Rounded as
+        // written: the order of two cells' rates has to be the same in every kernel
+        const T inv = arcp(w[0]), vx = tmul(w[1], inv), vy = tmul(w[2], inv);
+        const T p = tmul(gm1, tfma(T(-0.5), tfma(w[1], vx, tmul(w[2], vy)), w[3]));
         rmin = fmin(rmin, w[0]);
         pmin = fmin(pmin, p);
         // CFL rate beta^x / hx + beta^y / hy at the point
-        rate = nan_max(fabs(vx) * ihx + fabs(vy) * ihy + asqrt(gam * p * inv) * (ihx + ihy), rate);
+        const T c = asqrt(tmul(tmul(gam, p), inv));
+        rate = nan_max(tfma(c, tadd(ihx, ihy), tfma(fabs(vy), ihy, tmul(fabs(vx), ihx))), rate);
       });
       // the margins with some slack: limit_cells decides with sums in a fixed order
       const bool fails = active && eps > T(0) && eps_r > T(0) && (rmin < T(1.01) * eps_r || pmin < T(1.01) * eps);
@@ -1759,46 +1765,53 @@ struct Stage2D {
       } else {
         // The FP32 form's dt follows the digits of the rate at the point that gives the maximum, and next
         // to vacuum those digits depend on the order of the sum. So the factorised sums only choose the
-        // cell of each lane with the largest rate, and last_rate forms it again by the plain sum mode by
-        // mode (as limit_cells does for a cell that fails). Only the last stage's rate is used.
+        // cell with the largest rate of the whole mesh (of equal rates the lowest cell, so that the choice
+        // does not depend on the tiles), and the end of the step forms its rate by the plain sum mode by
+        // mode (top_rate; limit_cells does so for a cell that fails). Only the last stage's rate is used.
         if (!want_rate) return T(0);
-        if (active && !fails && rate > top.rest) {
-          top.rest = rate;
+        if (active && !fails && rate > top.rate) {
+          top.rate = rate;
           top.row = row;
         }
         return fails || rate != rate ? rate : T(0);
       }
     }
   }
-  // The end of an item (FP32 form): the plain rates of the lanes' cells, from the states just stored, if
-  // they are at least `below` (a part of u^n's rate, under which they will not be the maximum).
-  static __device__ __forceinline__ T last_rate(const Stage2DArgs& a, const TopRate& top, int xc, T below, T gam, T gm1) {
-    if (!__any_sync(0xffffffffu, top.rest >= below)) return top.rest;
-    T cell[NV][NM], lo[NV];
-    Store<PR, NV, NM, true>::load(a.uout, a.ncell, (long long)top.row * a.nx + xc, cell, lo);
-    const T plain = plain_rate(cell, gam, gm1, (T)a.hx, (T)a.hy);
-    return top.rest > T(0) ? plain : T(0);
-  }
-  // The largest CFL rate over the limiter's points of a cell, each point value summed mode by mode.
-  static __device__ __noinline__ T plain_rate(const T (&u)[NV][NM], T gam, T gm1, T hx, T hy) {
+  // The largest CFL rate over the limiter's points of a cell of state u, each point value summed mode by
+  // mode by a lane of its own. Called by a warp.
+  static __device__ __noinline__ T top_rate(const void* u, long long ncell, long long cell, T gam, T gm1, T hx, T hy) {
     const carr<T, NP_LIM * NM>& C = lim_table<K, BASIS, T>;
-    T rate = T(0);
-#pragma unroll 2
-    for (int i = 0; i < NP_LIM; ++i) {
+    T c[NV][NM], lo[NV], rate = T(0);
+    Store<PR, NV, NM, true>::load(u, ncell, cell, c, lo);
+#pragma unroll 1
+    for (int i = threadIdx.x & 31; i < NP_LIM; i += 32) {
       T w[NV];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) w[v] = u[v][0];
+      for (int v = 0; v < NV; ++v) w[v] = c[v][0];
 #pragma unroll
       for (int m = 1; m < NM; ++m) {
-        const T c = C[i * NM + m];
+        const T at = C[i * NM + m];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) w[v] = tfma(c, u[v][m], w[v]);
+        for (int v = 0; v < NV; ++v) w[v] = tfma(at, c[v][m], w[v]);
       }
       T bx, by, invH;
       bool ph;
       avg_params<EQ, 2>(w, gam, gm1, T(0), T(0), bx, by, invH, ph);
       rate = nan_max(bx / hx + by / hy, rate);
     }
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) rate = nan_max(__shfl_xor_sync(0xffffffffu, rate, o), rate);
+    return rate;
+  }
+  // The end of a step, once every cell of the state u is stored: the rate of the cell in sc->top_cell, which is
+  // cleared; 0 if there is none. Called by a warp.
+  static __device__ __forceinline__ T take_top_rate(DevScalars* sc, const void* u, long long ncell, T gam, T gm1, T hx,
+                                                    T hy) {
+    const unsigned long long key = *(const volatile unsigned long long*)&sc->top_cell;
+    if (key == 0ull) return T(0);
+    const T rate = top_rate(u, ncell, key_cell(key), gam, gm1, hx, hy);
+    if ((threadIdx.x & 31) == 0) *(volatile unsigned long long*)&sc->top_cell = 0ull;
     return rate;
   }
   // Admissibility margins, relative to the cell average in both precisions (as the oracle):
@@ -1908,10 +1921,19 @@ struct Stage2D {
     double my_rate = 0.0;
     T my_rate_t = T(0);
     bool my_ok = true;
+    unsigned long long my_top = 0ull;
     if (gw < (long long)a.nstrips * a.nchunks)
-      item(a, ctl.dt, (int)(gw % a.nstrips), (int)(gw / a.nstrips), ws, my_rate, my_rate_t, my_ok);
-    if constexpr (PR::MIXED) stage_end(a.sc, a.stage, ctl, a.cfl, my_rate_t, 1.0, my_ok, red);
-    else stage_end(a.sc, a.stage, ctl, a.cfl, my_rate, 1.0, my_ok, red);
+      item(a, ctl.dt, (int)(gw % a.nstrips), (int)(gw / a.nstrips), ws, my_rate, my_rate_t, my_ok, my_top);
+    if constexpr (TOP) {
+      fold_key(&a.sc->top_cell, my_top);
+      stage_end<true>(a.sc, a.stage, ctl, a.cfl, my_rate_t, 1.0, my_ok, red, [&]() -> double {
+        return (double)take_top_rate(a.sc, a.uout, a.ncell, (T)a.gamma, (T)(a.gamma - 1.0), (T)a.hx, (T)a.hy);
+      });
+    } else if constexpr (PR::MIXED) {
+      stage_end(a.sc, a.stage, ctl, a.cfl, my_rate_t, 1.0, my_ok, red);
+    } else {
+      stage_end(a.sc, a.stage, ctl, a.cfl, my_rate, 1.0, my_ok, red);
+    }
   }
 };
 

@@ -163,33 +163,58 @@ __device__ __forceinline__ StageCtl stage_begin(DevScalars* sc, int stage, doubl
   return stage_begin(sc, stage, cfl, [](int, const StageCtl&) {});
 }
 
+// A cell and a rate > 0 as one number that orders by the rate, and of equal rates by the lower cell
+// (cells are below 2^31, so no key is 0).
+__device__ __forceinline__ unsigned long long cell_key(float rate, long long cell) {
+  return ((unsigned long long)__float_as_uint(rate) << 32) | (unsigned)~(unsigned)cell;
+}
+__device__ __forceinline__ long long key_cell(unsigned long long key) { return (long long)(unsigned)~(unsigned)key; }
+// The warp's largest key, into *to. Called by all lanes.
+__device__ __forceinline__ void fold_key(unsigned long long* to, unsigned long long key) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32) == hi ? (unsigned)key : 0u);
+  if (hi != 0u && (threadIdx.x & 31) == 0) atomicMax(to, ((unsigned long long)hi << 32) | lo);
+}
+
 // Block-level end of a stage: publish non-physical flags; in the final stage also the rate max (my_rate
 // times `scale`, reduced in the stage's own arithmetic, scaled in FP64) and the last-block step advance.
-// Every thread of the block must call it (uses __syncthreads).
-template <class T>
+// Every thread of the block must call it (uses __syncthreads). LAST: last() runs in the first warp of the
+// last block, after every block's work, and returns (in lane 0) one more rate.
+template <bool LAST, class T, class F>
 __device__ __forceinline__ void stage_end(DevScalars* sc, int stage, const StageCtl& ctl, double cfl, T my_rate,
-                                          double scale, bool my_ok, T* red /* >= 32 words of shared memory */) {
+                                          double scale, bool my_ok, T* red /* >= 32 words of shared memory */,
+                                          F&& last) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
   T r = my_rate;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) r = nan_max(__shfl_xor_sync(0xffffffffu, r, o), r);
   if (lane == 0) red[wid] = r;
   const bool bad = __syncthreads_or(!my_ok) != 0;
-  if (threadIdx.x != 0) return;
-  if (bad) atomicOr(&sc->err, ERRB_NONPHYS);
+  if (threadIdx.x >= (LAST ? 32 : 1)) return;
+  if (bad && threadIdx.x == 0) atomicOr(&sc->err, ERRB_NONPHYS);
   if (stage != 2) return;
-  for (int w = 1; w < nw; ++w) r = nan_max(red[w], r);
   const long long st = ctl.step + 1;
-  atomic_max_nonneg(&sc->rate_bits[st & 1], (double)r * scale);
+  unsigned before = 0u;
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < nw; ++w) r = nan_max(red[w], r);
+    atomic_max_nonneg(&sc->rate_bits[st & 1], (double)r * scale);
+    __threadfence();
+    before = atomicAdd(&sc->blocks_done, 1u);
+  }
+  if constexpr (LAST) before = __shfl_sync(0xffffffffu, before, 0);
+  if (before != gridDim.x * gridDim.y - 1) return;
   __threadfence();
-  if (atomicAdd(&sc->blocks_done, 1u) != gridDim.x * gridDim.y - 1) return;
-  __threadfence();
+  if constexpr (LAST) {
+    const double more = last();
+    if (threadIdx.x != 0) return;
+    atomic_max_nonneg(&sc->rate_bits[st & 1], more);
+  }
   volatile DevScalars* vs = sc;
-  const unsigned err = vs->err, last = vs->is_last;
+  const unsigned err = vs->err, clipped = vs->is_last;
   const double t = vs->t, T_end = vs->T_end;
   const long long max_step = vs->max_step;
   if (err == 0u) {
-    const double tn = last ? T_end : t + ctl.dt;
+    const double tn = clipped ? T_end : t + ctl.dt;
     vs->t = tn;
     vs->step = st;
     vs->done = (tn >= T_end || st >= max_step) ? 1u : 0u;
@@ -198,6 +223,11 @@ __device__ __forceinline__ void stage_end(DevScalars* sc, int stage, const Stage
     vs->dt_cfl_step = st;
   }
   vs->blocks_done = 0u;
+}
+template <class T>
+__device__ __forceinline__ void stage_end(DevScalars* sc, int stage, const StageCtl& ctl, double cfl, T my_rate,
+                                          double scale, bool my_ok, T* red) {
+  stage_end<false>(sc, stage, ctl, cfl, my_rate, scale, my_ok, red, [] { return 0.0; });
 }
 
 // Hybrid limiter (Algorithm 1), one row of output cells of a warp: eta and the filter factors of the

@@ -53,3 +53,65 @@ def test_solvers_with_different_default_tiles_side_by_side(k, limiter):
     assert N.batch_run(solvers, 2, persistent=True) == 0
     for s in solvers:
         assert s.sync()[2] == 10
+
+
+def _limited(tile, k, kind, precision=N.PREC_FP32_MIXED):
+    s = N.Solver(dim=2, nx=90, ny=70, k=k, eq=N.EQ_EULER, bc=(N.BC_OUTFLOW,) * 4, precision=precision,
+                 tile_rows=tile[0], tile_warps=tile[1], positivity=1)
+    if kind == "quadrants":
+        s.set_initial(N.IC_QUADRANT2D, I.quadrant_params(1))
+    else:
+        # a stream whose waves run across the strips: the largest rate is met in every row, to rounding
+        x = (np.arange(90) + 0.5) / 90
+        rho = np.broadcast_to(1.0 + 0.2 * np.sin(6 * np.pi * x), (70, 90)).ravel()
+        u = np.zeros(s.shape)
+        u[0, 0], u[1, 0], u[2, 0], u[3, 0] = rho, 0.7 * rho, 0.3 * rho, 2.5 + 0.29 * rho
+        u[:, 1] = 0.01 * u[:, 0]
+        s.write_state(u)
+    return s
+
+
+# with the limiter in the FP32 form the rate that sets dt is summed again for the cells with the largest rates:
+# which they are must not follow the cut into tiles, nor how far a clipped step was
+@pytest.mark.parametrize("kind", ["quadrants", "stream"])
+@pytest.mark.parametrize("k", [1, 2, 3])
+def test_tile_shape_does_not_change_the_limited_result(k, kind):
+    def steps(tile):
+        s = _limited(tile, k, kind)
+        s.advance_steps(40)
+        s.advance_to(s.sync()[1] * 1.0101)              # ends on a clipped step
+        s.advance_steps(40)
+        assert s.sync()[0] == 0
+        out = s.read_state()
+        s.close()
+        return out
+    ref, t_ref = steps(TILES[0])
+    for tile in TILES[1:]:
+        u, t = steps(tile)
+        assert t == t_ref, tile
+        np.testing.assert_array_equal(u, ref, err_msg=str(tile))
+
+
+# the batched runs cut a class's meshes into chunks of their own
+@pytest.mark.parametrize("kind", ["quadrants", "stream"])
+@pytest.mark.parametrize("k", [1, 2, 3])
+@pytest.mark.parametrize("persistent", [False, True])
+def test_batched_limited_results_equal_solo(k, kind, persistent):
+    solo, batched = (_limited((0, 0), k, kind) for _ in range(2))
+    others = [_limited((0, 0), k, "quadrants") for _ in range(3)]
+    solo.advance_steps(30)
+    T = solo.sync()[1] * 1.0101
+    solo.advance_to(T)
+    clipped = solo.sync()[2]
+    solo.advance_steps(30)
+    for s in others:
+        s.set_target(T, 1 << 40)
+    batched.set_target(T, 1 << 40)
+    assert N.batch_run([batched] + others, clipped, persistent=persistent) == 0
+    assert batched.sync() == (0, T, clipped)
+    batched.set_target(float("inf"), 1 << 40)
+    assert N.batch_run([batched] + others, 30, persistent=persistent) == 0
+    u, t = solo.read_state()
+    ub, tb = batched.read_state()
+    assert tb == t
+    np.testing.assert_array_equal(ub, u)
