@@ -319,9 +319,12 @@ constexpr carr<T, limiter_points(K) * Modes<K, BASIS>::NM> limiter_values() {
   }
   return t;
 }
-// (In global memory: a warp reads them a lane per point, and the constant cache serves one address at a time.)
+// Once in global memory, for a warp that reads them a lane per point, and once in constant memory, which
+// serves one address at a time, for lanes that go through the points together.
 template <int K, int BASIS, class T>
 __device__ const carr<T, limiter_points(K) * Modes<K, BASIS>::NM> lim_table = limiter_values<K, BASIS, T>();
+template <int K, int BASIS, class T>
+__constant__ __align__(16) carr<T, limiter_points(K) * Modes<K, BASIS>::NM> lim_const = limiter_values<K, BASIS, T>();
 
 // OE = true: the OEDG form of the damping (DG_FILTER_OEDG): the kernel stores u~ unfiltered with the
 // jump sums A_v(l) and the reductions of OedgOut, and the OEDG filter kernel applies the damping.
@@ -1737,9 +1740,20 @@ struct Stage2D {
         const T c = asqrt(tmul(tmul(gam, p), inv));
         rate = nan_max(tfma(c, tadd(ihx, ihy), tfma(fabs(vy), ihy, tmul(fabs(vx), ihx))), rate);
       });
-      // the margins with some slack: limit_cells decides with sums in a fixed order
-      const bool fails = active && eps > T(0) && eps_r > T(0) && (rmin < T(1.01) * eps_r || pmin < T(1.01) * eps);
-      const unsigned mask = __ballot_sync(0xffffffffu, fails);
+      // the margins with some slack: limit_cells and limit_lanes decide with sums in a fixed order
+      const bool thin = rmin < T(1.01) * eps_r;
+      bool fails = active && eps > T(0) && eps_r > T(0) && (thin || pmin < T(1.01) * eps);
+      unsigned mask = __ballot_sync(0xffffffffu, fails);
+      if (mask) {
+        // a cell without higher modes has nothing to limit, whatever its margin
+        bool varies = false;
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+          for (int m = 1; m < NM; ++m) varies = varies || uo[v][m] != T(0);
+        fails = fails && varies;
+        mask = __ballot_sync(0xffffffffu, fails);
+      }
       if (mask) {
         const int lane = threadIdx.x & 31;
         if (fails) {
@@ -1750,7 +1764,12 @@ struct Stage2D {
         }
         __syncwarp();
         T th1 = T(1), th2 = T(1);
-        limit_cells(mask, ws, slot, eps_r, eps, gam, gm1, hx, hy, th1, th2, rate);
+        if (__popc(mask) < LIMIT_LANES) {
+          limit_cells(mask, ws, slot, eps_r, eps, gam, gm1, hx, hy, th1, th2, rate);
+        } else if (fails) {
+          limit_lanes(ws, slot, thin, want_rate, eps_r, eps, gam, gm1, hx, hy, th1, th2, rate);
+        }
+        __syncwarp();
         if (fails) {
 #pragma unroll
           for (int m = 1; m < NM; ++m) {
@@ -1830,6 +1849,114 @@ struct Stage2D {
     eps_r = ub[0] < eps_r ? ub[0] : eps_r;
     eps = ub[0] < eps ? ub[0] : eps;
     eps = pbar < eps ? pbar : eps;
+  }
+  // theta_1, theta_2 and the limited cell's rate, each failing lane for its own cell (in row slot `slot`), two
+  // points at a time, with the sums of limit_cells; thin: the density may fail, rated: the rate is wanted.
+  // For rows where many cells fail, as in cold flows: where p_bar is below 1e-3 (rho_bar + |E_bar|) the margin
+  // is p_bar itself, which a smooth cell meets only to rounding. Bound by issue: a pass over the points and
+  // 30 evaluations for each that a smaller theta_2 does not cover yet. From LIMIT_LANES failing cells of a warp
+  // on it is the faster one (4, 8, 16 within 1 % but for mesh edges, where 16 loses). us per step at 512^2,
+  // rho = 1, p = 1e-6, FP32 form, degree 1 / 2 / 3, limit_cells alone -> with this: at rest 410 / 768 / 2121 ->
+  // 146 / 299 / 1334, in uniform motion 521 / 1034 / 4207 -> 152 / 283 / 1336, waves in the stream 1350 / 1537 /
+  // 5496 -> 583 / 1062 / 4088 (a warm state, where few cells fail: 109 / 172 / 599).
+  static constexpr int LIMIT_LANES = 8;
+  static __device__ __noinline__ void limit_lanes(T* ws, int slot, bool thin, bool rated, T eps_r, T eps, T gam, T gm1,
+                                                  T hx, T hy, T& th1_, T& th2_, T& rate_) {
+    const carr<T, NP_LIM * NM>& C = lim_const<K, BASIS, T>;
+    const int lane = threadIdx.x & 31;
+    VG u[NG][NM];
+    sfor<NG>([&](auto G_) {
+      constexpr int g = decltype(G_)::value;
+#pragma unroll
+      for (int m = 0; m < NM; ++m) u[g][m] = gslot<g>(ws, slot, m, lane);
+    });
+    T ub[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) ub[v] = *slot_ptr(ws, slot, v, 0, lane);
+    auto scale = [&](VG x, T f) -> VG {
+      if constexpr (PACK) return f2{tmul(x.x, f), tmul(x.y, f)};
+      else return tmul(x, f);
+    };
+    auto values = [&](int i, T (&w)[NV]) {
+      VG x[NG];
+#pragma unroll
+      for (int g = 0; g < NG; ++g) {
+        x[g] = u[g][0];
+#pragma unroll
+        for (int m = 1; m < NM; ++m) {
+          if constexpr (PACK) x[g] = vmad(u[g][m], C[i * NM + m], x[g]);
+          else x[g] = tfma(C[i * NM + m], u[g][m], x[g]);
+        }
+      }
+      sfor<NG>([&](auto G_) {
+        constexpr int g = decltype(G_)::value;
+        if constexpr (PACK) {
+          w[2 * g] = x[g].x;
+          w[2 * g + 1] = x[g].y;
+        } else {
+          w[g] = x[g];
+        }
+      });
+    };
+    auto rate_at = [&](const T (&w)[NV]) -> T {
+      T bx, by, invH;
+      bool ph;
+      avg_params<EQ, 2>(w, gam, gm1, T(0), T(0), bx, by, invH, ph);
+      return bx / hx + by / hy;
+    };
+    if (thin) {
+      T low = ub[0];
+#pragma unroll 1
+      for (int i = 0; i < NP_LIM; ++i) {
+        T w[NV];
+        values(i, w);
+        low = fmin(low, w[0]);
+      }
+      if (low < eps_r) {
+        const T th1 = (ub[0] - eps_r) / (ub[0] - low);
+        th1_ = th1;
+#pragma unroll
+        for (int m = 1; m < NM; ++m) {
+          if constexpr (PACK) u[0][m].x = tmul(u[0][m].x, th1);
+          else u[0][m] = tmul(u[0][m], th1);
+        }
+      }
+    }
+    T th2 = T(1), rate = T(0);
+    // a point that fails: its segment is solved only if theta_2 so far is not enough for it
+    auto solve = [&](const T (&w)[NV]) {
+      T x[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) x[v] = ub[v] + th2 * (w[v] - ub[v]);
+      if (th2 < T(1) && pressure_of<NV>(x, gm1) >= eps) return;
+      th2 = fmin(th2, pp_segment<NV>(ub, w, eps, gm1));
+    };
+#pragma unroll 1
+    for (int i = 0; i < NP_LIM; i += 2) {
+      T a[NV], b[NV];
+      values(i, a);
+      values(i + 1 < NP_LIM ? i + 1 : i, b);                      // (the last point of an odd number twice)
+      const T pa = pressure_of<NV>(a, gm1), pb = pressure_of<NV>(b, gm1);
+      if (rated) rate = nan_max(rate_at(a), nan_max(rate_at(b), rate));
+      if (pa < eps) solve(a);
+      if (pb < eps) solve(b);
+    }
+    if (th2 < T(1) && rated) {
+#pragma unroll
+      for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int m = 1; m < NM; ++m) u[g][m] = scale(u[g][m], th2);
+      rate = T(0);
+#pragma unroll 1
+      for (int i = 0; i < NP_LIM; i += 2) {
+        T a[NV], b[NV];
+        values(i, a);
+        values(i + 1 < NP_LIM ? i + 1 : i, b);
+        rate = nan_max(rate_at(a), nan_max(rate_at(b), rate));
+      }
+    }
+    th2_ = th2;
+    rate_ = rate;
   }
   // theta_1, theta_2 and the limited cell's rate for the cells of the lanes in mask, which hold their
   // coefficients in row slot `slot`: lane i evaluates point i (and i + 32) of each cell and solves for
