@@ -8,6 +8,7 @@
 // fixed launch sequence (6 kernels, 1D: 2) that is captured once into a CUDA graph and replayed; dt, t and
 // the stop condition live on the device.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -89,6 +90,8 @@ dg_status dgk::validate_config(const dg_mesh* m, int k, int eq, const dg_filter_
   if (p->precision != DG_PREC_FP64 && p->precision != DG_PREC_FP32_MIXED) return DG_ERR_ARG;
   if (!(p->cfl > 0.0) || !(p->gamma > 1.0)) return DG_ERR_ARG;
   if ((long long)m->nx * (m->dim == 2 ? m->ny : 1) > (1LL << 31)) return DG_ERR_UNSUPPORTED;
+  // the 2D row march counts two rows past the last, and the columns of its last strip, in 32 bits
+  if (m->dim == 2 && (m->nx > INT_MAX - 27 || m->ny > INT_MAX - 4)) return DG_ERR_UNSUPPORTED;
   if (p->hybrid && (!p->enabled || p->positivity)) return DG_ERR_UNSUPPORTED;
   if (p->filter_kind < DG_FILTER_JUMP || p->filter_kind > DG_FILTER_OEDG) return DG_ERR_ARG;
   if (p->hybrid && p->filter_kind != DG_FILTER_JUMP) return DG_ERR_UNSUPPORTED;
@@ -258,7 +261,7 @@ TileShape dgk::tile_shape(const StageLauncher& L, int nstrips, int ny, bool fp64
       long long nch = (long long)w * nsm / nstrips;
       nch = nch < 1 ? 1 : (nch > ny ? ny : nch);
       const int H = rows > 0 ? (rows < ny ? rows : ny) : (int)((ny + nch - 1) / nch);
-      const double t = tile_cost((long long)nstrips * ((ny + H - 1) / H), H, wpb, bps * wpb, nsm, fp64);
+      const double t = tile_cost((long long)nstrips * tiles_of(ny, H), H, wpb, bps * wpb, nsm, fp64);
       if (cost < 0.0 || t < cost) {
         cost = t;
         best = TileShape{H, wpb};
@@ -271,7 +274,7 @@ TileShape dgk::tile_shape(const StageLauncher& L, int nstrips, int ny, bool fp64
 
 static dg_status setup_launch(dg_solver* s, int tile_rows, int tile_warps) {
   if (s->dim == 1) {
-    s->nwarps1d = (s->mesh.nx + STRIP_OUT - 1) / STRIP_OUT;
+    s->nwarps1d = (int)tiles_of(s->mesh.nx, STRIP_OUT);
     // the whole step in one launch, unless a second kernel has to run between the stages
     s->whole_step = !s->hybrid && !s->geom.oedg;
     if (s->whole_step) {
@@ -302,7 +305,7 @@ static dg_status setup_launch(dg_solver* s, int tile_rows, int tile_warps) {
                                                      : stage2d_f32_launcher(s->k, s->eq, s->basis)));
   if (!s->L.launch) return DG_ERR_UNSUPPORTED;
   const int nx = s->mesh.nx, ny = s->mesh.ny;
-  s->nstrips = (nx + STRIP_OUT - 1) / STRIP_OUT;
+  s->nstrips = (int)tiles_of(nx, STRIP_OUT);
   const TileShape tile = tile_shape(s->L, s->nstrips, ny, s->prec == PREC_F64, tile_rows, tile_warps);
   if (tile.warps < 1) return DG_ERR_UNSUPPORTED;
   const int wpb = tile.warps, H = tile.rows;
@@ -311,7 +314,7 @@ static dg_status setup_launch(dg_solver* s, int tile_rows, int tile_warps) {
   s->block = 32 * wpb;
   s->smem = 256 + s->L.slot_bytes_per_warp * wpb;
   s->H = H;
-  s->nchunks = (ny + H - 1) / H;
+  s->nchunks = (int)tiles_of(ny, H);
   long long nw = (long long)s->nstrips * s->nchunks;
   s->grid = (unsigned)((nw + wpb - 1) / wpb);
   return DG_OK;

@@ -217,7 +217,7 @@ template <class S>
 __device__ __forceinline__ void step1d_tile(const Stage1DArgs& a, Step1DShared<S>& sh, long long tile,
                                             typename S::T& speed, bool& ok) {
   BlockLink<typename S::T> link{sh.link, (int)(threadIdx.x >> 5), STEP1D_THREADS / 32};
-  const typename S::Place pl = S::place(a, (int)(tile * STEP1D_OUT) - STEP_HALO, (int)threadIdx.x, STEP1D_THREADS, STEP_HALO);
+  const typename S::Place pl = S::place(a, tile * STEP1D_OUT - STEP_HALO, (int)threadIdx.x, STEP1D_THREADS, STEP_HALO);
   typename S::T un[S::NV][S::NM], unlo[S::NV];
   S::ST::load(a.un, a.ncell, pl.cell, un, unlo);
   S::step_tile(a, sh.coef, (typename S::T)sh.dt, pl, link, un, unlo, speed, ok);
@@ -687,7 +687,7 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       I.bcx = s->mesh.bc[0];
       I.bcy = s->dim == 2 ? s->mesh.bc[2] : 0;
       I.H = s->dim == 2 ? s->H : 1;
-      I.nstrips = s->dim == 2 ? s->nstrips : (int)((s->mesh.nx + STEP1D_OUT - 1) / STEP1D_OUT);
+      I.nstrips = s->dim == 2 ? s->nstrips : (int)tiles_of(s->mesh.nx, STEP1D_OUT);
       I.nchunks = s->dim == 2 ? s->nchunks : 1;
       I.strips = I.nstrips;
       I.limited = s->dim == 2 && s->positivity ? s->k : 0;
@@ -771,7 +771,7 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
         long long items = 0;
         for (int i = 0; i < cls_count[c]; ++i) {
           const int hi = own[i] ? (h < I[i].ny ? h : I[i].ny) : I[i].H;
-          items += (long long)I[i].nstrips * ((I[i].ny + hi - 1) / hi);
+          items += (long long)I[i].nstrips * tiles_of(I[i].ny, hi);
         }
         const int fit = best > 0 ? best : 1;
         const long long per = (items + (long long)nsm * fit - 1) / ((long long)nsm * fit);
@@ -785,7 +785,7 @@ static dg_status batch_run(dg_solver* const* solvers, int n, long long steps, bo
       for (int i = 0; i < cls_count[c]; ++i) {
         if (!own[i]) continue;
         I[i].H = rows < I[i].ny ? rows : I[i].ny;
-        I[i].nchunks = (I[i].ny + I[i].H - 1) / I[i].H;
+        I[i].nchunks = (int)tiles_of(I[i].ny, I[i].H);
       }
     }
     if (c < 3 && persistent) {

@@ -11,6 +11,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include "cell_index.h"
 #include "dg_tables.cuh"
 
 namespace dgk {

@@ -89,7 +89,7 @@ Step1DGrid step1d_grid(const StageLauncher& L, long long n) {
   for (int nt : {32, 64, 128, STEP_THREADS}) {
     const int bps = L.blocks_per_sm(nt, 0);
     if (bps < 1) continue;
-    const long long tiles = (n + nt - 2 * STEP_HALO - 1) / (nt - 2 * STEP_HALO);
+    const long long tiles = tiles_of(n, nt - 2 * STEP_HALO);
     const long long c = (((tiles + nsm - 1) / nsm) * (nt / 32) + 3) / 4;
     if (cost >= 0 && c >= cost) continue;
     cost = c;

@@ -400,7 +400,7 @@ struct Stage1D {
   static __device__ void item(const Stage1DArgs& a, double dtd, long long strip, T& my_speed, bool& my_ok) {
     const int lane = threadIdx.x & 31;
     const Coef k = coef_of_stage(a.c1 * dtd, a.inv_h_d, a.c0, df{a.c0_hi, a.c0_lo});
-    const Place pl = place(a, (int)strip * STRIP_OUT - 2, lane, 32, 2);
+    const Place pl = place(a, strip * STRIP_OUT - 2, lane, 32, 2);
     T u[NV][NM], lo[NV], un[NV][NM], unlo[NV];
     ST::load(a.uin, a.ncell, pl.cell, u, lo);
     if (a.stage > 0) ST::load(a.un, a.ncell, pl.cell, un, unlo);
@@ -448,16 +448,17 @@ struct Stage1D {
     }
   }
   // Lane i of `lanes` cells from x0, with `halo` cells on each side that are not its output.
-  static __device__ __forceinline__ Place place(const Stage1DArgs& a, int x0, int i, int lanes, int halo) {
-    const int nx = a.nx, x = x0 + i;
-    const bool per = a.bc == BC_PERIODIC;
+  static __device__ __forceinline__ Place place(const Stage1DArgs& a, long long x0, int i, int lanes, int halo) {
+    const int nx = a.nx;
+    const unsigned c = column_of(x0) + (unsigned)i;
+    const bool per = a.bc == BC_PERIODIC, inside = column_inside(c, nx);
     Place p;
-    p.cell = per ? ((x % nx) + nx) % nx : (x < 0 ? 0 : (x >= nx ? nx - 1 : x));
-    p.ghost = !per && (x < 0 || x >= nx);
-    p.take_right = x == -1;
-    p.take_left = x == nx;
+    p.cell = cell_column(c, nx, per);
+    p.ghost = !per && !inside;
+    p.take_right = c == COLUMN0 - 1;
+    p.take_left = c == COLUMN0 + (unsigned)nx;
     p.edge = !per && (x0 < 0 || x0 + lanes > nx);
-    p.own = i >= halo && i < lanes - halo && x >= 0 && x < nx;
+    p.own = i >= halo && i < lanes - halo && inside;
     return p;
   }
 
@@ -637,7 +638,7 @@ struct Stage1D {
     const int out = (int)blockDim.x - 2 * STEP_HALO;
     // the first tile's state is on its way while the step control is read
     long long tile = blockIdx.x;
-    Place pl = place(a, (int)(tile * out) - STEP_HALO, (int)threadIdx.x, (int)blockDim.x, STEP_HALO);
+    Place pl = place(a, tile * out - STEP_HALO, (int)threadIdx.x, (int)blockDim.x, STEP_HALO);
     T un[NV][NM], unlo[NV];
     ST::load(a.un, a.ncell, pl.cell, un, unlo);
     const StageCtl ctl = stage_begin(a.sc, 0, a.cfl,
@@ -651,7 +652,7 @@ struct Stage1D {
       step_tile(a, coef, dt, pl, link, un, unlo, my_speed, my_ok);
       tile += gridDim.x;
       if (tile >= a.nwarps) break;
-      pl = place(a, (int)(tile * out) - STEP_HALO, (int)threadIdx.x, (int)blockDim.x, STEP_HALO);
+      pl = place(a, tile * out - STEP_HALO, (int)threadIdx.x, (int)blockDim.x, STEP_HALO);
       ST::load(a.un, a.ncell, pl.cell, un, unlo);
     }
     stage_end(a.sc, 2, ctl, a.cfl, my_speed, a.inv_h_d, my_ok, red);

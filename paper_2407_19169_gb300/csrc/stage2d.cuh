@@ -998,7 +998,7 @@ struct Stage2D {
     {
       const int x = strip * STRIP_OUT - 2 + lane;
       const bool perx = a.bcx == BC_PERIODIC, pery = a.bcy == BC_PERIODIC;
-      const int xc = perx ? ((x % nx) + nx) % nx : (x < 0 ? 0 : (x >= nx ? nx - 1 : x));
+      const int xc = perx ? wrap_column(x, nx) : (x < 0 ? 0 : (x >= nx ? nx - 1 : x));
       // outflow: columns and rows outside the mesh are ghost cells holding the constant state equal
       // to the adjacent interior cell's average (stage input for the fluxes, u~ for the jumps)
       const bool gcol = !perx && (x < 0 || x >= nx);
@@ -1006,7 +1006,7 @@ struct Stage2D {
       const bool edge_strip = !perx && (xw < 0 || xw + 31 >= nx);
       const bool out_lane = lane >= 2 && lane < 2 + STRIP_OUT && x >= 0 && x < nx;
       const int yb = chunk * a.H;
-      const int ye = min(yb + a.H, ny);
+      const int ye = (int)min((unsigned)yb + (unsigned)a.H, (unsigned)ny);
 
       T topPrev[NQ][NV];
 #pragma unroll
