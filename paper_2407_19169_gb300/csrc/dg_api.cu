@@ -463,7 +463,7 @@ static dg_status reset_control(dg_solver* s, double t) {
   s->h_sc->max_step = 1LL << 62;
   CK(cudaMemcpyAsync(s->sc, s->h_sc, sizeof(DevScalars), cudaMemcpyHostToDevice, s->stream));
   CK(launch_rate(s->geom, s->buf[0], s->sc, 0, s->stream));
-  s->launches += 1;
+  s->launches += rate_launches(s->geom);
   s->h_step = 0;
   return DG_OK;
 }

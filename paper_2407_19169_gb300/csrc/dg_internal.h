@@ -68,6 +68,7 @@ dg_status check_device(char* why, size_t why_len);
 cudaError_t launch_project(const AuxGeom& g, int ic, const double* prm, int nprm, int nq,
                            double* canon_out, cudaStream_t s);
 cudaError_t launch_rate(const AuxGeom& g, const void* state, DevScalars* sc, int slot, cudaStream_t s);
+int rate_launches(const AuxGeom& g);   // kernels of one launch_rate
 cudaError_t launch_to_storage(const AuxGeom& g, const double* canon, void* state, cudaStream_t s);
 cudaError_t launch_from_storage(const AuxGeom& g, const void* state, double* canon, cudaStream_t s);
 cudaError_t launch_mass(const AuxGeom& g, const void* state, double* partials, double* out, cudaStream_t s);

@@ -337,5 +337,6 @@ cudaError_t launch_rate(const AuxGeom& g, const void* state, DevScalars* sc, int
   k.evaluate<<<blocks, 256, 0, s>>>(g, state, sc, slot);
   return cudaGetLastError();
 }
+int rate_launches(const AuxGeom& g) { return rate_kernels_of(g).bound ? 2 : 1; }
 
 }  // namespace dgk
