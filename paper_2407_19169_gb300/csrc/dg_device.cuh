@@ -440,7 +440,8 @@ __device__ __forceinline__ void llf2d_twice(const T* uL, const T* uR, T* fh, T g
 __device__ __forceinline__ float keep_max(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ double keep_max(double a, double b) { return nan_max(a, b); }
 
-// Cell-average quantities for the filter and the CFL rate: beta^x, beta^y, 1/Hbar.
+// Cell-average quantities for the filter and the CFL rate: beta^x, beta^y, 1/Hbar. A wave speed or 1/Hbar
+// that underflows to zero is physical: it damps nothing and sets no dt.
 template <int EQ, int DIM, class T>
 __device__ __forceinline__ void avg_params(const T* ub, T gamma, T gm1, T ax, T ay, T& bx, T& by,
                                            T& invH, bool& physical) {
@@ -462,7 +463,7 @@ __device__ __forceinline__ void avg_params(const T* ub, T gamma, T gm1, T ax, T 
     bx = fabs(vel) + c;
     by = T(0);
     invH = ub[0] * arcp(ub[2] + p);
-    physical = pos_finite(ub[0]) && pos_finite(p) && pos_finite(bx) && pos_finite(invH);
+    physical = pos_finite(ub[0]) && pos_finite(p) && !not_finite(bx) && !not_finite(invH);
   } else {
     T inv = arcp(ub[0]);
     T vx = ub[1] * inv, vy = ub[2] * inv;
@@ -471,7 +472,7 @@ __device__ __forceinline__ void avg_params(const T* ub, T gamma, T gm1, T ax, T 
     bx = fabs(vx) + c;
     by = fabs(vy) + c;
     invH = ub[0] * arcp(ub[3] + p);
-    physical = pos_finite(ub[0]) && pos_finite(p) && pos_finite(bx) && pos_finite(by) && pos_finite(invH);
+    physical = pos_finite(ub[0]) && pos_finite(p) && !not_finite(bx) && !not_finite(by) && !not_finite(invH);
   }
 }
 

@@ -42,7 +42,7 @@ static __device__ __forceinline__ double rate_of(const AuxGeom& g, const double*
       invH = ub[0] * (1.0 / (ub[3] + p));
     }
     bx = fabs(vx) + c;
-    phys = pos_finite(ub[0]) && pos_finite(p) && pos_finite(bx) && (DIM == 1 || pos_finite(by)) && pos_finite(invH);
+    phys = pos_finite(ub[0]) && pos_finite(p) && !not_finite(bx) && (DIM == 1 || !not_finite(by)) && !not_finite(invH);
   } else {
     avg_params<EQ, DIM>(ub, g.gamma, g.gamma - 1.0, g.ax, g.ay, bx, by, invH, phys);
   }

@@ -84,3 +84,22 @@ def _step_time(k, precision, n, kind):
                                                    (N.PREC_FP64, 256, "inflow", 6.0)])
 def test_cold_flows_cost_little_more_than_warm_ones(precision, n, kind, most):
     assert _step_time(2, precision, n, kind) <= most * _step_time(2, precision, n, "warm")
+
+
+@pytest.mark.parametrize("dim", [1, 2])
+@pytest.mark.parametrize("k", [1, 2, 3])
+def test_wave_speed_below_the_smallest_float_is_physical(dim, k):
+    # gamma p / rho = 3.9e-39: the FP32 form's wave speed at rest is zero, 1 / H = 1e38 is finite
+    n = 64
+    s = N.Solver(dim=dim, nx=n, ny=8 if dim == 2 else 1, k=k, eq=N.EQ_EULER, bc=(N.BC_OUTFLOW,) * 4,
+                 precision=N.PREC_FP32_MIXED)
+    u = np.zeros(s.shape)
+    cold = np.arange(u.shape[2]) % n < n // 2
+    u[0, 0] = 1e4
+    u[-1, 0] = np.where(cold, 2.8e-35, 1.0) / 0.4
+    s.write_state(u)
+    s.step()
+    v, t = s.read_state()
+    far = np.arange(u.shape[2]) % n < n // 2 - 6                 # a step reaches six cells
+    assert t > 0.0 and np.isfinite(v).all()
+    np.testing.assert_allclose(v[:, 0][:, far], u[:, 0][:, far], rtol=1e-6)
