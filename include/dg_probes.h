@@ -32,6 +32,10 @@ DG_API int dg_probe_transform(int variant, long long ncell, int reps, double* ms
  * satisfied ends, reports, and leaves the context usable. */
 DG_API int dg_probe_wait_timeout(unsigned poll_limit, unsigned* status, double* ms);
 
+/* The FP64 functions of the stage kernels on n host values x, each through a GPU thread: fn 0 = reciprocal,
+ * 1 = square root, 2 = damping factor exp(x) of x <= 0 (chosen per warp of 32 consecutive values). */
+DG_API int dg_probe_fp64(int fn, long long n, const double* x, double* y);
+
 #ifdef __cplusplus
 }
 #endif

@@ -29,7 +29,7 @@ EXPORTED = ["dg_status_string", "dg_last_error", "dg_params_default", "dg_worksp
             "dg_read_state_device", "dg_step", "dg_advance_to", "dg_advance_steps", "dg_sync", "dg_mass",
             "dg_dims", "dg_kernel_launches", "dg_destroy", "dg_step_noalloc", "dg_set_target",
             "dg_batch_run", "dg_batch_run_persistent", "dg_probe_fma", "dg_probe_transform",
-            "dg_probe_wait_timeout"]
+            "dg_probe_wait_timeout", "dg_probe_fp64"]
 
 
 class Mesh(C.Structure):
@@ -95,6 +95,7 @@ def load():
         "dg_probe_fma": (I, [I, I, dp]),
         "dg_probe_transform": (I, [I, LL, I, dp, dp]),
         "dg_probe_wait_timeout": (I, [C.c_uint, P(C.c_uint), dp]),
+        "dg_probe_fp64": (I, [I, LL, dp, dp]),
     }
     for name, (res, args) in sig.items():
         f = getattr(L, name)

@@ -24,8 +24,9 @@ UNITS = [(u, u.replace(".cu", ".o"), []) for u in
         [("dg_batch.cu", "dg_batch_k%d.o" % k, ["-DDG_BATCH_K=%d" % k]) for k in (1, 2, 3)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -prec-div=false / -prec-sqrt=false: single-precision division and square root by the hardware
-# approximations (a couple of ulp). They act only on FP32 arithmetic (the FP32 form's stage math);
-# FP64 and the double-float cell averages are untouched.
+# approximations (a couple of ulp). They act only on FP32 arithmetic (the FP32 form's stage math); the
+# double-float cell averages are untouched. FP64's own reciprocal, root and damping exponential, within an
+# ulp, are in csrc/dg_device.cuh.
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-prec-div=false", "-prec-sqrt=false",
          "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]
 

@@ -193,10 +193,11 @@ __device__ __forceinline__ float arcp(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// FP64: the FP64 pipe issues one warp instruction every 16 cycles, and the library's correctly rounded
-// division and square root take about 8 and 10 of them. From the hardware's 20-bit approximation r one
-// third-order Newton-Householder step gives 1/x = r (1 + e + e^2 + O(e^3)), e = 1 - x r, to about an
-// ulp in 3 instructions.
+// FP64: an FP64 warp instruction holds its quarter of the SM for 64 cycles, and the library's correctly
+// rounded division and square root take about 8 and 10 of them. From the hardware's 20-bit approximation r
+// one third-order Newton-Householder step gives 1/x = r (1 + e + e^2 + O(e^3)), e = 1 - x r, in 3
+// instructions, at most one ulp from the correctly rounded value for 2^-1021 <= |x| < 2^1021
+// (dg_probe_fp64). No result for zero, subnormals and infinities.
 __device__ __forceinline__ double arcp(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -209,8 +210,9 @@ __device__ __forceinline__ float asqrt(float x) {
   return r;
 }
 // FP64: from y ~ 1/sqrt(x) (20 bits) and g = x y, sqrt(x) = g (1 - e)^(-1/2) with e = 1 - g y, by the
-// binomial series to second order (the next term is 5/16 e^3): 5 instructions, about an ulp. Zeros,
-// subnormals and negative arguments (NaN) take the library's function.
+// binomial series to second order (the next term is 5/16 e^3): 5 instructions, at most one ulp from the
+// correctly rounded value (dg_probe_fp64). Below 2^-1021 (zeros, subnormals, negative arguments) the
+// library's function; infinity gives NaN, which no caller takes for physical either.
 __device__ __forceinline__ double asqrt(double x) {
   if (__double2hiint(x) < 0x00200000) return sqrt(x);
   double y;
@@ -233,8 +235,10 @@ __device__ __forceinline__ bool pos_finite(float x) { return x > 0.f && isfinite
 
 // Damping factors f[l] = exp(x[l]), l = 1..N-1, of x <= 0 that decreases with l. FP64: where the solution is
 // smooth the arguments are tiny, and if all of the warp's are, the Taylor polynomial of degree 6
-// (|x| < 2^-9: the next term is below 2^-75) or 10 (|x| < 2^-4: below 2^-69) is exact to rounding in 6 or
-// 10 instructions instead of the function's 15 or more. Called by all lanes of the warp.
+// (|x| < 2^-9: the next term is below 2^-75) or 10 (|x| < 2^-4: below 2^-69) takes 6 or 10 instructions
+// instead of the function's 15 or more, at most one ulp from it (dg_probe_fp64). Called by all lanes of the
+// warp: which of the three a cell gets depends on the cells that share its warp, so its last bit may
+// differ with the 1D tile's width (step1d_grid: the SM count) and with the 2D strip.
 template <int N>
 __device__ __forceinline__ void exp_damp(const float (&x)[N], float (&f)[N]) {
 #pragma unroll

@@ -10,6 +10,7 @@
 #include <stdint.h>
 
 #include "../../include/dg_probes.h"
+#include "dg_device.cuh"
 
 namespace {
 
@@ -202,6 +203,22 @@ __global__ void mma_transform_kernel(const float* __restrict__ u, float* __restr
   }
 }
 
+// ---- the stage kernels' FP64 functions ------------------------------------------------------------
+__global__ void __launch_bounds__(128) fp64_kernel(int fn, long long n, const double* x, double* y) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const double a = x[i < n ? i : n - 1];
+  double r;
+  if (fn == 2) {                                              // a vote of whole warps
+    const double e[2] = {0.0, a};
+    double f[2];
+    dgk::exp_damp(e, f);
+    r = f[1];
+  } else {
+    r = fn == 0 ? dgk::arcp(a) : dgk::asqrt(a);
+  }
+  if (i < n) y[i] = r;
+}
+
 // relative L1 of a float result against the FP64 reference: partial sums per block
 __global__ void err_kernel(const float* f, const double* r, long long total, double* acc) {
   __shared__ double sn[256], sd[256];
@@ -331,4 +348,19 @@ extern "C" int dg_probe_transform(int variant, long long ncell, int reps, double
   cudaFree(acc);
   cudaStreamDestroy(st);
   return status;
+}
+
+extern "C" int dg_probe_fp64(int fn, long long n, const double* x, double* y) {
+  if (!x || !y || fn < 0 || fn > 2 || n < 1 || n > (1ll << 24)) return -1;
+  double* d = nullptr;
+  const size_t bytes = sizeof(double) * (size_t)n;
+  if (cudaMalloc(&d, 2 * bytes) != cudaSuccess) return -2;
+  cudaError_t e = cudaMemcpy(d, x, bytes, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    fp64_kernel<<<(unsigned)((n + 127) / 128), 128>>>(fn, n, d, d + n);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(y, d + n, bytes, cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return e == cudaSuccess ? 0 : -6;
 }
