@@ -10,8 +10,7 @@
 // The array: NOALLOC_SCRATCH_BYTES (32 MiB + 256 B) of static device memory, reserved on every GPU
 // that loads this library until the process exits. Host code cannot use the array's name as a
 // device address, so the first call on each device (with that device current) sets the device up
-// once: it checks that the device is an sm_103 GPU, copies the Gauss rules that the initial
-// CFL-rate kernel reads into the device's constant memory, and looks the array's address up with
+// once: it checks that the device is an sm_103 GPU and looks the array's address up with
 // cudaGetSymbolAddress, caching it; make that first call outside any stream capture. The cached
 // address belongs to the device's context of that moment: after a cudaDeviceReset in the same
 // process it is stale, so no further call may be made on that device. All calls share the array
@@ -82,10 +81,9 @@ extern "C" dg_status dg_step_noalloc(const dg_mesh* m, int k, int eq, const dg_f
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return DG_ERR_CUDA;
   if (!g_scratch_addr[dev]) {
-    // once per device: an sm_103 GPU, the Gauss rules in constant memory, the array's address
+    // once per device: an sm_103 GPU, the array's address
     char why[128];
     if (check_device(why, sizeof(why)) != DG_OK) return DG_ERR_CUDA;
-    if (aux_init_tables() != cudaSuccess) return DG_ERR_CUDA;
     void* ptr = nullptr;
     if (cudaGetSymbolAddress(&ptr, g_noalloc_scratch) != cudaSuccess || !ptr) return DG_ERR_CUDA;
     g_scratch_addr[dev] = ptr;

@@ -395,7 +395,8 @@ struct Stage1D {
     return OE ? (2 * r + 1) / cfact(r) * (1 << r) : (r == 0 ? 1.0 : (double)(r * (r + 1) * (1 << r)));
   }
 
-  // One stage of a 32-cell strip (28 output cells) of one instance, step size dtd. The output cells'
+  // One stage of a 32-cell strip (28 output cells) of one instance, step size dtd (the hybrid limiter and
+  // the OEDG form, neither of which runs with the positivity limiter). The output cells'
   // largest wave speed (the CFL rate times h) and physicality are folded into my_speed and my_ok.
   static __device__ void item(const Stage1DArgs& a, double dtd, long long strip, T& my_speed, bool& my_ok) {
     const int lane = threadIdx.x & 31;
@@ -414,14 +415,10 @@ struct Stage1D {
     T bx, eta = T(0);
     bool phys;
     cell_stage<true>(a, k, a.stage == 0, (T)dtd, pl, link, u, lo, un, unlo, bx, phys, eta);
-    T rate = T(0);
-    if constexpr (EQ == EQ_EULER) {
-      if (a.positivity) rate = limit_and_rate(u, pl.own, (T)a.gamma, (T)(a.gamma - 1.0));
-    }
     if (pl.own) {
       ST::store(a.uout, a.ncell, pl.cell, u, lo);
       if (!phys) my_ok = false;
-      my_speed = nan_max(nan_max(bx, rate), my_speed);
+      my_speed = nan_max(bx, my_speed);
     }
     if (a.hybrid) hybrid_max(a.hyb, pl.own ? eta : T(0));
     if constexpr (OE) {

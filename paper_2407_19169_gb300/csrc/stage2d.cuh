@@ -31,13 +31,13 @@ namespace dgk {
 
 // Mesh and physics constants of a 2D stage, computed once by stage2d_consts (on the host for a
 // single solve, so that the kernel reads them from its parameter space instead of holding them in
-// registers): powers of 2/h for physical derivatives, the filter's per-order jump weights (the jump
-// filter's m(m+1) h^m, or the OEDG form's (2m+1)/m! h^(m-1), with the trapezoid's 1/2), 1/h, gamma,
-// gamma - 1 and the advection velocity.
+// registers): products of powers of 2/h for physical derivatives, the filter's per-order jump weights
+// (the jump filter's m(m+1) h^m, or the OEDG form's (2m+1)/m! h^(m-1), with the trapezoid's 1/2), 1/h,
+// gamma, gamma - 1 and the advection velocity.
 template <class T>
 struct Consts2D {
-  T px[4], py[4], wx[7], wy[7];
-  T pxy[16], pxy2[16];   // (2/h_x)^a1 (2/h_y)^a2 at [a1 * 4 + a2], and twice that
+  T wx[7], wy[7];
+  T pxy2[16];            // 2 (2/h_x)^a1 (2/h_y)^a2 at [a1 * 4 + a2]
   T pxyk2[16];           // pxy2 times P_k^(k) for each order that is the degree k (folded top derivatives)
   T ihx, ihy, gam, gm1, ax, ay;
 };
@@ -80,13 +80,8 @@ __host__ __device__ inline void consts2d_fill(Consts2D<T>& c, double hx, double 
     px[r] = px[r - 1] * (2.0 / hx);
     py[r] = py[r - 1] * (2.0 / hy);
   }
-  for (int r = 0; r < 4; ++r) {
-    c.px[r] = (T)px[r];
-    c.py[r] = (T)py[r];
-  }
   for (int a1 = 0; a1 < 4; ++a1)
     for (int a2 = 0; a2 < 4; ++a2) {
-      c.pxy[a1 * 4 + a2] = (T)(px[a1] * py[a2]);
       c.pxy2[a1 * 4 + a2] = (T)(2.0 * px[a1] * py[a2]);
       const double top = dend(1, k, k);
       c.pxyk2[a1 * 4 + a2] = (T)(2.0 * px[a1] * py[a2] * (a1 == k ? top : 1.0) * (a2 == k ? top : 1.0));
@@ -870,10 +865,9 @@ struct Stage2D {
   }
 
   // |value at +1| + |value at -1| of the R-th derivative of the jump polynomial with coefficients
-  // c[0..K] of normal order NO across an x-edge (DIR = 0) or a y-edge (DIR = 1), times f, into acc.
+  // c[0..K] of normal order NO across an x-edge (DIR = 0) or a y-edge (DIR = 1), times f2x / 2, into acc.
   template <int DIR, int NO, int R, class VT>
-  static __device__ __forceinline__ void corner_pair(const VT (&c)[K + 1], typename vtraits<VT>::S f,
-                                                     typename vtraits<VT>::S f2x, VT& acc) {
+  static __device__ __forceinline__ void corner_pair(const VT (&c)[K + 1], typename vtraits<VT>::S f2x, VT& acc) {
     using S = typename vtraits<VT>::S;
     constexpr bool HE = DIR == 0 ? xt(NO, R, 0) : yt(NO, R, 0);
     constexpr bool HO = DIR == 0 ? xt(NO, R, 1) : yt(NO, R, 1);
@@ -901,8 +895,7 @@ struct Stage2D {
   // Right vertical edge of the cell w: per total order m, sum over |alpha| = m of
   // f_alpha (|jump at the bottom corner| + |jump at the top corner|) into sv[m].
   template <class VT>
-  static __device__ __forceinline__ void vertical_jumps(const VT (&w)[NM], VT (&sv)[LMAX + 1], const T* pxy,
-                                                        const T* pxy2) {
+  static __device__ __forceinline__ void vertical_jumps(const VT (&w)[NM], VT (&sv)[LMAX + 1], const T* pxy2) {
     sfor<K + 1>([&](auto A1_) {
       constexpr int a1 = decltype(A1_)::value;
       VT W[K + 1];
@@ -917,7 +910,7 @@ struct Stage2D {
       sfor<K + 1>([&](auto A2_) {
         constexpr int a2 = decltype(A2_)::value;
         if constexpr (TB::alpha_ok(a1, a2) && (xt(a1, a2, 0) || xt(a1, a2, 1)))
-          corner_pair<0, a1, a2>(W, pxy[a1 * 4 + a2], pxy2[a1 * 4 + a2], sv[a1 + a2]);
+          corner_pair<0, a1, a2>(W, pxy2[a1 * 4 + a2], sv[a1 + a2]);
       });
     });
   }
@@ -925,7 +918,7 @@ struct Stage2D {
   // The horizontal edge between the cell below (wb, its top) and the cell above (wa, its bottom).
   template <class VT>
   static __device__ __forceinline__ void horizontal_jumps(const VT (&wa)[NM], const VT (&wb)[NM], VT (&sh)[LMAX + 1],
-                                                          const T* pxy, const T* pxy2) {
+                                                          const T* pxy2) {
     sfor<K + 1>([&](auto A2_) {
       constexpr int a2 = decltype(A2_)::value;
       VT V[K + 1];
@@ -941,7 +934,7 @@ struct Stage2D {
       sfor<K + 1>([&](auto A1_) {
         constexpr int a1 = decltype(A1_)::value;
         if constexpr (TB::alpha_ok(a1, a2) && (yt(a2, a1, 0) || yt(a2, a1, 1)))
-          corner_pair<1, a2, a1>(V, pxy[a1 * 4 + a2], pxy2[a1 * 4 + a2], sh[a1 + a2]);
+          corner_pair<1, a2, a1>(V, pxy2[a1 * 4 + a2], sh[a1 + a2]);
       });
     });
   }
@@ -977,11 +970,9 @@ struct Stage2D {
     const df dfx = df_from_double(0.5 * c1dt * ihx);
     const df dfy = df_from_double(0.5 * c1dt * ihy);
     const df dfc0 = df_from_double(a.c0);
-    // powers of 2/h for physical derivatives; weights of the m-th derivative jumps (with the 1/2 of
-    // the trapezoidal rule over an edge's two corners): the jump filter's m(m+1) h^m, or the OEDG
-    // form's (2m+1)/m! h^m, each direction divided by its own h (Section 2.1's form)
-    const T* px = KC.px;
-    const T* py = KC.py;
+    // weights of the m-th derivative jumps (with the 1/2 of the trapezoidal rule over an edge's two
+    // corners): the jump filter's m(m+1) h^m, or the OEDG form's (2m+1)/m! h^m, each direction divided
+    // by its own h (Section 2.1's form)
     const T* wx = KC.wx;
     const T* wy = KC.wy;
     // OEDG reductions of this lane's output cells: sum of the averages, largest / smallest value at
@@ -1425,8 +1416,8 @@ struct Stage2D {
             // whose guards fail only in the first iteration: -> 0.482 ms. Those writes go to a row
             // slot that the partial stage value of row yb overwrites before it is read. Unguarding
             // the partial stage value itself as well was slower, 0.497 ms)
-            if (PACK || need_v) vertical_jumps(w1, sv, KC.pxy, FOLD ? KC.pxyk2 : KC.pxy2);
-            horizontal_jumps(w1, w2, sh, KC.pxy, FOLD ? KC.pxyk2 : KC.pxy2);
+            if (PACK || need_v) vertical_jumps(w1, sv, FOLD ? KC.pxyk2 : KC.pxy2);
+            horizontal_jumps(w1, w2, sh, FOLD ? KC.pxyk2 : KC.pxy2);
             VG av = z, shc = z;
 #pragma unroll
             for (int l = 0; l <= LMAX; ++l) {
