@@ -229,6 +229,11 @@ __device__ __forceinline__ bool pos_finite(double x) {
   const long long b = __double_as_longlong(x);
   return b > 0 && b < 0x7ff0000000000000ll;
 }
+// 0 <= x < infinity (not for -0): one comparison of unsigned bits
+__device__ __forceinline__ bool zero_or_pos_finite(double x) {
+  return (unsigned long long)__double_as_longlong(x) < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool zero_or_pos_finite(float x) { return isfinite(x); }
 __device__ __forceinline__ bool not_finite(double x) { return abs_bits(x) >= 0x7ff0000000000000ll; }
 __device__ __forceinline__ bool not_finite(float x) { return !isfinite(x); }
 __device__ __forceinline__ bool pos_finite(float x) { return x > 0.f && isfinite(x); }
@@ -467,7 +472,7 @@ __device__ __forceinline__ void avg_params(const T* ub, T gamma, T gm1, T ax, T 
     bx = fabs(vel) + c;
     by = T(0);
     invH = ub[0] * arcp(ub[2] + p);
-    physical = pos_finite(ub[0]) && pos_finite(p) && !not_finite(bx) && !not_finite(invH);
+    physical = pos_finite(ub[0]) && pos_finite(p) && zero_or_pos_finite(bx) && zero_or_pos_finite(invH);
   } else {
     T inv = arcp(ub[0]);
     T vx = ub[1] * inv, vy = ub[2] * inv;
@@ -476,7 +481,7 @@ __device__ __forceinline__ void avg_params(const T* ub, T gamma, T gm1, T ax, T 
     bx = fabs(vx) + c;
     by = fabs(vy) + c;
     invH = ub[0] * arcp(ub[3] + p);
-    physical = pos_finite(ub[0]) && pos_finite(p) && !not_finite(bx) && !not_finite(by) && !not_finite(invH);
+    physical = pos_finite(ub[0]) && pos_finite(p) && zero_or_pos_finite(bx) && zero_or_pos_finite(by) && zero_or_pos_finite(invH);
   }
 }
 
