@@ -225,8 +225,9 @@ int dgk::device_sms() {
 // cost about three rows' work in the FP32 form and two in FP64 (their guarded parts are skipped). What
 // a row costs depends on the warps that share the SM. FP32 form: a quarter of an SM that holds one warp
 // runs at its latency, two take 1.5 times as long (2048^2 Q2: 5400 and 4030 cycles per row and warp).
-// FP64: the pipe serves the whole SM, and four warps fill it. More warps than are resident run in
-// rounds. So few rows per chunk where the mesh leaves quarters idle, and many where it fills them.
+// FP64: an instruction holds its quarter's pipe for 64 cycles, so up to four warps run side by side and
+// more share the quarters; one warp a quarter is counted as filling it, though it keeps the pipe 76 % busy
+// (Q2 512^2), since the row slots of an eighth warp do not fit. More warps than are resident run in rounds. So few rows per chunk where the mesh leaves quarters idle, and many where it fills them.
 double dgk::tile_cost(long long items, int rows, int warps, int resident, int nsm, bool fp64) {
   const long long blocks = (items + warps - 1) / warps;
   const long long w = ((blocks + nsm - 1) / nsm) * warps;

@@ -78,7 +78,11 @@ StageLauncher step1d_launcher(int K, int EQ, int PREC) {
 // issue slots and the FP64 pipe belong to the quarters of an SM (an FP64 warp instruction holds its
 // quarter for 64 cycles), so the time follows the warps of the fullest quarter: the smallest NT of 32,
 // 64, 128 and 256 with the fewest (a few cells spread over the SMs, many take wide tiles with little
-// halo), then at most the resident blocks, which loop over their tiles.
+// halo), then at most the resident blocks, which loop over their tiles. The FP32 form also waits at the
+// block's barriers, which the rule leaves out. Euler, us per step with 32 / 64 / 128 / 256 threads, the
+// rule's choice in brackets: FP32 form P2 10^4 cells (9.3) 8.3 8.3 9.2, 65536 26.0 13.0 (11.3) 11.3,
+// 2 10^5 34.8 20.1 (18.2) 18.5, 10^6 82.6 66.4 59.9 (60.4), P3 65536 26.9 14.4 (12.4) 12.4; FP64 P3 65536
+// 222 182 (160) 159.
 Step1DGrid step1d_grid(const StageLauncher& L, long long n) {
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||

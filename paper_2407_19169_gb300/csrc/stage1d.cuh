@@ -626,8 +626,8 @@ struct Stage1D {
   // state is read and written once per step (one launch per stage moved it 8 times and paid three
   // launches), and the step control is paid once. Bound by instruction issue in the FP32 form and by the
   // FP64 pipe (64 cycles a warp instruction on a quarter of an SM) in FP64. Per step, before and after:
-  // Burgers P2 200 cells FP64 27.7 -> 15.4 us, Euler P3 65536 cells FP64 230 -> 165, FP32 form 31.2 ->
-  // 13.3, Euler P2 1 M cells FP32 form 156 -> 59, with the limiter 179 -> 68.
+  // Burgers P2 200 cells FP64 27.7 -> 15.0 us, Euler P3 65536 cells FP64 230 -> 160, FP32 form 31.2 ->
+  // 12.4, Euler P2 1 M cells FP32 form 156 -> 60, with the limiter 179 -> 69.
   static __device__ void run_step(const Stage1DArgs& a) {
     __shared__ T link_words[LINK_BUFFERS][LINK_WARPS][LINK_WORDS];
     __shared__ Coef coef[3];

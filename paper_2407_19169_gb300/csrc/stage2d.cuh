@@ -198,9 +198,10 @@ struct Store {
     }
   }
   // Rows staged through shared memory by asynchronous copies, up to nine modes (the rows of more would
-  // take the shared memory of their row slots, and the persistent batched kernels, COH, share an SM
-  // between classes): a warp's buffer holds VECS float4 planes of 32 cells and, with an even number of
-  // modes, a float2 plane per pair of variables; each lane copies and reads the words of its own cell.
+  // take the shared memory of their row slots), but not in the persistent batched kernels (COH): with Q2's
+  // rows staged there (all its copies go through L2) a batch of twelve uneven solves took 35.8 ms instead of
+  // 22.0, the same states. A warp's buffer holds PVECS float4 planes of 32 cells per pair of variables
+  // and, with an even number of modes, a float2 plane; each lane copies and reads its own cell's words.
   static constexpr bool STAGED = PAIRED && NM <= 9 && !COH;
   static constexpr int PVECS = 1 + (NM - 1) / 2;              // float4 planes of a pair
   static constexpr bool TAIL = ((NM - 1) & 1) != 0;
@@ -1706,11 +1707,12 @@ struct Stage2D {
   //
   // Bound by instruction issue. Nearly every cell is admissible, so one sum-factorised pass over the
   // points takes the smallest density and pressure and the rate together (a step of a 1024^2 Q2 solve
-  // with the limiter 819 -> 550 us, without it 425; Q3 at 512^2 702 -> 572, without it 486; FP64 Q2 at
+  // with the limiter 819 -> 508 us, without it 387; Q3 at 512^2 702 -> 595, without it 479; FP64 Q2 at
   // 128^2 4137 -> 2970; before: a dense sum per point, once for the density, once for the pressure and
-  // once for the rate); the cells of a warp that fail are limited one after the other by
-  // the whole warp, a lane per point (limit_cells), so that a strip along a near-vacuum front, whose
-  // every row has such cells, does not hold its launch up. Called by all lanes of the warp; ws, slot:
+  // once for the rate, and rows not yet staged); the few cells of a warp that fail are limited one
+  // after the other by the whole warp, a lane per point (limit_cells), so that a strip along a near-vacuum
+  // front, whose every row has such cells, does not hold its launch up; many of them with a lane each
+  // (limit_lanes). Called by all lanes of the warp; ws, slot:
   // a row slot that holds nothing any more (the cells are passed through it).
   static __device__ __forceinline__ T limit_and_rate(T (&uo)[NV][NM], bool active, bool want_rate, T* ws, int slot,
                                                      T gam, T gm1, T ihx, T ihy, T hx, T hy, int row, TopRow& top) {

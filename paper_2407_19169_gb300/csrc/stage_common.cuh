@@ -10,7 +10,10 @@
 // dt never travels to the host.
 //
 // Protocol on DevScalars (no spin-waits anywhere):
-//   - every stage kernel returns at once if done or err is set (values fixed during the launch);
+//   - every stage kernel returns at once if done or err is set. done is fixed during a launch; err is
+//     set by any block that ends with a non-physical cell, and a block that begins after it then returns
+//     without counting itself, so blocks_done may stay non-zero after an error until the next written
+//     state clears the scalars (a solve in error takes no further step);
 //   - stage 0: every block takes the same dt from (t, T_end) and cfl / rate, which the last block of
 //     the previous step left in dt_cfl (the first step divides by rate_bits[step & 1] itself); block 0
 //     publishes dt and is_last;
