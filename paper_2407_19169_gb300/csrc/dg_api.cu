@@ -242,8 +242,10 @@ double dgk::tile_cost(long long items, int rows, int warps, int resident, int ns
 // one: Q2 FP32 form 64^2 102 -> 46 us, 128^2 102 -> 55, 256^2 104 -> 83, with the limiter 128^2 122 -> 60;
 // Q3 128^2 280 -> 122; FP64 Q2 128^2 2225 -> 856, P3 160^2 3046 -> 1318; from 512^2 on the same.
 TileShape dgk::tile_shape(const StageLauncher& L, int nstrips, int ny, bool fp64, int rows, int warps) {
-  // at most the row slots that fit in 200 KB of shared memory
-  int most = (int)((200 * 1024 - 256) / L.slot_bytes_per_warp);
+  // at most the row slots that fit in a block's shared memory (227 KB, 1 KB of it for static variables): eight
+  // warps of Q2's FP32 form, with its staged rows, take 221 KB (with 200 KB a tile of 128 rows x 8 warps ran
+  // as 7 warps in two rounds: 2048^2 2.60 ms a step instead of 1.35)
+  int most = (int)((226 * 1024 - 256) / L.slot_bytes_per_warp);
   if (most > 8) most = 8;
   if (most < 1) return TileShape{0, 0};
   // the kernel's shared-memory limit is one for all its launches: always that of the largest block, so

@@ -1,6 +1,8 @@
 """The 2D tile shape (rows per warp item, warps per block) changes only the schedule: every shape
 the autotuner may pick, 1-warp blocks and the library's default schedule (0, 0) give bitwise the
 same state."""
+import time
+
 import numpy as np
 import pytest
 
@@ -115,3 +117,23 @@ def test_batched_limited_results_equal_solo(k, kind, persistent):
     ub, tb = batched.read_state()
     assert tb == t
     np.testing.assert_array_equal(ub, u)
+
+
+@pytest.mark.parametrize("limiter", [0, 1])
+def test_eight_warps_cost_no_more_than_two_blocks_of_four(limiter):
+    # 2048^2 in 128 rows: 1184 items, a round of 1216 resident warps with either block; seven-warp blocks take two
+    def step_time(warps):
+        s = N.Solver(dim=2, nx=2048, ny=2048, k=2, eq=N.EQ_EULER, bc=(N.BC_OUTFLOW,) * 4, positivity=limiter,
+                     precision=N.PREC_FP32_MIXED, tile_rows=128, tile_warps=warps)
+        s.set_initial(N.IC_QUADRANT2D, I.quadrant_params(1))
+        best = np.inf
+        for _ in range(4):                                    # the first pass warms up
+            t0 = time.perf_counter()
+            s.advance_steps(8)
+            assert s.sync()[0] == 0
+            best = min(best, time.perf_counter() - t0)
+        s.close()
+        print("%d warps: %.1f us per step" % (warps, best / 8 * 1e6))
+        return best
+
+    assert step_time(8) <= 1.3 * step_time(4)
