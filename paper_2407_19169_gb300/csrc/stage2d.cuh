@@ -1736,39 +1736,26 @@ struct Stage2D {
       // the margins with some slack: limit_cells and limit_lanes decide with sums in a fixed order
       const bool thin = rmin < T(1.01) * eps_r;
       bool fails = active && eps > T(0) && eps_r > T(0) && (thin || pmin < T(1.01) * eps);
-      unsigned mask = __ballot_sync(0xffffffffu, fails);
+      const unsigned mask = __ballot_sync(0xffffffffu, fails);
       if (mask) {
-        // a cell without higher modes has nothing to limit, whatever its margin
-        bool varies = false;
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-#pragma unroll
-          for (int m = 1; m < NM; ++m) varies = varies || uo[v][m] != T(0);
-        fails = fails && varies;
-        mask = __ballot_sync(0xffffffffu, fails);
-      }
-      if (mask) {
-        const int lane = threadIdx.x & 31;
         if (fails) {
+          const int lane = threadIdx.x & 31;
 #pragma unroll
           for (int v = 0; v < NV; ++v)
 #pragma unroll
             for (int m = 0; m < NM; ++m) *slot_ptr(ws, slot, v, m, lane) = uo[v][m];
         }
         __syncwarp();
-        T th1 = T(1), th2 = T(1);
-        if (__popc(mask) < LIMIT_LANES) {
-          limit_cells(mask, ws, slot, eps_r, eps, gam, gm1, hx, hy, th1, th2, rate);
-        } else if (fails) {
-          limit_lanes(ws, slot, thin, want_rate, eps_r, eps, gam, gm1, hx, hy, th1, th2, rate);
-        }
+        const Limited c = limit_row(fails, ws, slot, thin, want_rate, eps_r, eps, gam, gm1, hx, hy, rate);
         __syncwarp();
+        fails = c.limited;
+        rate = c.rate;
         if (fails) {
 #pragma unroll
           for (int m = 1; m < NM; ++m) {
-            uo[0][m] *= th1;
+            uo[0][m] *= c.th1;
 #pragma unroll
-            for (int v = 0; v < NV; ++v) uo[v][m] *= th2;
+            for (int v = 0; v < NV; ++v) uo[v][m] *= c.th2;
           }
         }
       }
@@ -1788,6 +1775,32 @@ struct Stage2D {
         return fails || rate != rate ? rate : T(0);
       }
     }
+  }
+  // The failing lanes' cells of a row (in row slot `slot`), their rates before in `rate`. A cell without higher
+  // modes has nothing to limit, whatever its margin. Out of line as a whole: with the choice between the two
+  // paths in limit_and_rate every row paid for it (Q2 1024^2, 8 steps: 4.69 ms a pass, so 4.65). Called by a warp.
+  struct Limited {
+    T th1, th2, rate;
+    bool limited;
+  };
+  static __device__ __noinline__ Limited limit_row(bool fails, T* ws, int slot, bool thin, bool rated, T eps_r, T eps,
+                                                   T gam, T gm1, T hx, T hy, T rate) {
+    const int lane = threadIdx.x & 31;
+    bool varies = false;
+    if (fails) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int m = 1; m < NM; ++m) varies = varies || *slot_ptr(ws, slot, v, m, lane) != T(0);
+    }
+    Limited c{T(1), T(1), rate, varies};
+    const unsigned mask = __ballot_sync(0xffffffffu, varies);
+    if (__popc(mask) < LIMIT_LANES) {
+      if (mask) limit_cells(mask, ws, slot, eps_r, eps, gam, gm1, hx, hy, c.th1, c.th2, c.rate);
+    } else if (varies) {
+      limit_lanes(ws, slot, thin, rated, eps_r, eps, gam, gm1, hx, hy, c.th1, c.th2, c.rate);
+    }
+    return c;
   }
   // The largest CFL rate over the limiter's points of a cell of state u, each point value summed mode by
   // mode by a lane of its own. Called by a warp.
